@@ -109,6 +109,8 @@ struct lbm_ctx {
     int cur = 0;                  // f[cur] holds the current state
     void *q = nullptr;            // potential field of the current pass
     bool fused = false;           // FP32 single-pass step in use
+    bool wide = false;            // FP64-arithmetic two-pass step by block sums in use (wide_step.cu)
+    double *sums = nullptr;       // its block sums
     void *qpad[2] = {nullptr, nullptr};  // padded potential of f[0] / f[1] (fused path)
     bool qpad_valid = false;      // qpad[cur] holds the potential of f[cur]
     int seg_rows = 0;             // rows per CTA segment of the fused path (0: automatic)
@@ -260,28 +262,47 @@ cudaError_t timed_launch(lbm_ctx *c, int slot, Fn fn, int kernels = 1) {
     return cudaSuccess;
 }
 
-// One time step: potential of f[cur] into q, then force/collide/stream into f[1-cur].
-template <typename T>
-cudaError_t step_once(lbm_ctx *c, const Model<T> &m) {
-    const T *f = (const T *)c->f[c->cur];
-    T *g = (T *)c->f[1 - c->cur];
-    cudaError_t e = timed_launch(c, 0, [&] { return launch_potential<T>(m, is_sc(c), f, (T *)c->q, c->err, c->stream); });
+// The two passes in FP64 arithmetic of a state stored as TS: by block sums
+// where the context has them, else by the direct stencil.
+cudaError_t wide_potential(lbm_ctx *c, const Model<double> &m, const double *f, double *q, cudaStream_t s) {
+    return c->wide ? launch_wide_potential<double>(m, is_sc(c), is_cdm(c), f, q, c->sums, c->err, s)
+                   : launch_potential<double>(m, is_sc(c), f, q, c->err, s);
+}
+cudaError_t wide_potential(lbm_ctx *c, const Model<double> &m, const float *f, double *q, cudaStream_t s) {
+    return c->wide ? launch_wide_potential<float>(m, is_sc(c), is_cdm(c), f, q, c->sums, c->err, s)
+                   : launch_potential_mixed(m, is_sc(c), f, q, c->err, s);
+}
+cudaError_t wide_collide(lbm_ctx *c, const Model<double> &m, const double *f, const double *q, double *g, cudaStream_t s) {
+    return c->wide ? launch_wide_collide<double>(m, is_sc(c), is_cdm(c), f, q, c->sums, g, s)
+                   : launch_collide<double>(m, is_sc(c), is_cdm(c), f, q, g, s);
+}
+cudaError_t wide_collide(lbm_ctx *c, const Model<double> &m, const float *f, const double *q, float *g, cudaStream_t s) {
+    return c->wide ? launch_wide_collide<float>(m, is_sc(c), is_cdm(c), f, q, c->sums, g, s)
+                   : launch_collide_mixed(m, is_sc(c), is_cdm(c), f, q, g, s);
+}
+
+// One time step in FP64 arithmetic, f stored as TS (float: FP32 lattices off
+// the single-pass kernel): potential of f[cur] into q, then
+// force/collide/stream into f[1-cur].
+template <typename TS>
+cudaError_t step_once_wide(lbm_ctx *c, const Model<double> &m) {
+    const TS *f = (const TS *)c->f[c->cur];
+    cudaError_t e = timed_launch(c, 0, [&] { return wide_potential(c, m, f, (double *)c->q, c->stream); });
     if (e != cudaSuccess) return e;
-    e = timed_launch(c, 1, [&] { return launch_collide<T>(m, is_sc(c), is_cdm(c), f, (const T *)c->q, g, c->stream); });
+    e = timed_launch(c, 1, [&] { return wide_collide(c, m, f, (const double *)c->q, (TS *)c->f[1 - c->cur], c->stream); });
     if (e != cudaSuccess) return e;
     if (c->timing) c->tm.steps += 1;
     c->cur = 1 - c->cur;
     return cudaSuccess;
 }
 
-// One time step of an FP32 lattice in the two-pass form: FP32 distributions,
-// FP64 arithmetic and an FP64 potential field (see lbm_kernels.cu).
-cudaError_t step_once_mixed(lbm_ctx *c, const Model<double> &m) {
+// The same in FP32 arithmetic (LBM_FLAG_F32_ARITH).
+cudaError_t step_once_f32(lbm_ctx *c, const Model<float> &m) {
     const float *f = (const float *)c->f[c->cur];
     float *g = (float *)c->f[1 - c->cur];
-    cudaError_t e = timed_launch(c, 0, [&] { return launch_potential_mixed(m, is_sc(c), f, (double *)c->q, c->err, c->stream); });
+    cudaError_t e = timed_launch(c, 0, [&] { return launch_potential<float>(m, is_sc(c), f, (float *)c->q, c->err, c->stream); });
     if (e != cudaSuccess) return e;
-    e = timed_launch(c, 1, [&] { return launch_collide_mixed(m, is_sc(c), is_cdm(c), f, (const double *)c->q, g, c->stream); });
+    e = timed_launch(c, 1, [&] { return launch_collide<float>(m, is_sc(c), is_cdm(c), f, (const float *)c->q, g, c->stream); });
     if (e != cudaSuccess) return e;
     if (c->timing) c->tm.steps += 1;
     c->cur = 1 - c->cur;
@@ -318,28 +339,26 @@ cudaError_t step_fused(lbm_ctx *c, const Model<float> &m) {
 // Density and Eq. 11 velocity of the current state, in the arithmetic of the
 // lattice's step: FP32 for FP32 lattices on the single-pass kernel (or with
 // LBM_FLAG_F32_ARITH), FP64 for the other FP32 lattices (the mixed kernels).
-template <typename T>
-cudaError_t moments_into(lbm_ctx *c, T *r, T *vx, T *vy) {
-    Model<T> m = model_of<T>(c);
-    const T *f = (const T *)c->f[c->cur];
-    cudaError_t e = launch_potential<T>(m, is_sc(c), f, (T *)c->q, c->err, c->stream);
-    if (e != cudaSuccess) return e;
-    return launch_moments<T>(m, is_sc(c), is_cdm(c), f, (const T *)c->q, r, vx, vy, c->stream);
-}
-template <>
-cudaError_t moments_into<float>(lbm_ctx *c, float *r, float *vx, float *vy) {
-    if (c->fused || (c->p.flags & LBM_FLAG_F32_ARITH)) {
-        Model<float> mf = model_of<float>(c);
-        const float *f = (const float *)c->f[c->cur];
-        cudaError_t e = launch_potential<float>(mf, is_sc(c), f, (float *)c->q, c->err, c->stream);
-        if (e != cudaSuccess) return e;
-        return launch_moments<float>(mf, is_sc(c), is_cdm(c), f, (const float *)c->q, r, vx, vy, c->stream);
+template <typename TS>
+cudaError_t moments_into(lbm_ctx *c, TS *r, TS *vx, TS *vy) {
+    const TS *f = (const TS *)c->f[c->cur];
+    if constexpr (std::is_same_v<TS, float>) {
+        if (c->fused || (c->p.flags & LBM_FLAG_F32_ARITH)) {
+            Model<float> mf = model_of<float>(c);
+            cudaError_t e = launch_potential<float>(mf, is_sc(c), f, (float *)c->q, c->err, c->stream);
+            if (e != cudaSuccess) return e;
+            return launch_moments<float>(mf, is_sc(c), is_cdm(c), f, (const float *)c->q, r, vx, vy, c->stream);
+        }
     }
     Model<double> m = model_of<double>(c);
-    const float *f = (const float *)c->f[c->cur];
-    cudaError_t e = launch_potential_mixed(m, is_sc(c), f, (double *)c->q, c->err, c->stream);
+    double *q = (double *)c->q;
+    cudaError_t e = wide_potential(c, m, f, q, c->stream);
     if (e != cudaSuccess) return e;
-    return launch_moments_mixed(m, is_sc(c), is_cdm(c), f, (const double *)c->q, r, vx, vy, c->stream);
+    if (c->wide) return launch_wide_moments<TS>(m, is_sc(c), is_cdm(c), f, q, c->sums, r, vx, vy, c->stream);
+    if constexpr (std::is_same_v<TS, float>)
+        return launch_moments_mixed(m, is_sc(c), is_cdm(c), f, q, r, vx, vy, c->stream);
+    else
+        return launch_moments<double>(m, is_sc(c), is_cdm(c), f, q, r, vx, vy, c->stream);
 }
 
 // Three fields of scratch and, past them, the 8-byte word of the host-array
@@ -445,6 +464,22 @@ void free_tape(lbm_ctx *c) {
     c->tape_steps = -1;
 }
 
+// The two passes of the tape's forward steps on explicit buffers, in the
+// precision of the lattice.  (The recompute on the tape's stream and the
+// forward on the context's share the block sums: the sweep runs between an
+// event after the context's work and one before it goes on.)
+template <typename T>
+cudaError_t tape_potential(lbm_ctx *c, const Model<T> &m, const void *f, void *q, cudaStream_t s) {
+    if constexpr (std::is_same_v<T, double>) return wide_potential(c, m, (const double *)f, (double *)q, s);
+    else return launch_potential<T>(m, is_sc(c), (const T *)f, (T *)q, c->err, s);
+}
+template <typename T>
+cudaError_t tape_collide(lbm_ctx *c, const Model<T> &m, const void *f, const void *q, void *g, cudaStream_t s) {
+    if constexpr (std::is_same_v<T, double>)
+        return wide_collide(c, m, (const double *)f, (const double *)q, (double *)g, s);
+    else return launch_collide<T>(m, is_sc(c), is_cdm(c), (const T *)f, (const T *)q, (T *)g, s);
+}
+
 // One forward step from state `src` to `dst` (explicit buffers).  Single-pass
 // path: qsrc holds the padded stencil field of src (valid on entry) and qdst
 // receives that of dst.  Two-pass path: the potential of src is formed into
@@ -458,9 +493,9 @@ cudaError_t tape_step(lbm_ctx *c, const Model<T> &m, const void *src, void *dst,
             return launch_fused_step(m, is_sc(c), is_cdm(c), (const float *)src, (const float *)qsrc, (float *)dst,
                                      (float *)qdst, c->err, seg_rows_of(c), c->stream, true, rec, rev);
     }
-    cudaError_t e = launch_potential<T>(m, is_sc(c), (const T *)src, (T *)qsrc, c->err, c->stream);
+    cudaError_t e = tape_potential<T>(c, m, src, qsrc, c->stream);
     if (e != cudaSuccess) return e;
-    return launch_collide<T>(m, is_sc(c), is_cdm(c), (const T *)src, (const T *)qsrc, (T *)dst, c->stream);
+    return tape_collide<T>(c, m, src, qsrc, dst, c->stream);
 }
 
 template <typename T>
@@ -636,10 +671,9 @@ lbm_status tape_backward(lbm_ctx *c, const T *grad_rhoT, T *grad_rho0, double *g
         }
         const void *cur = c->ckpt[k];
         for (int t = t0; t < t1 && r == cudaSuccess; ++t) {
-            r = launch_potential<T>(m, is_sc(c), (const T *)cur, (T *)segqf(sl, t - t0), c->err, s);
+            r = tape_potential<T>(c, m, cur, segqf(sl, t - t0), s);
             if (r == cudaSuccess && t < t1 - 1) {
-                r = launch_collide<T>(m, is_sc(c), is_cdm(c), (const T *)cur, (const T *)segqf(sl, t - t0),
-                                      (T *)segf(sl, t - t0), s);
+                r = tape_collide<T>(c, m, cur, segqf(sl, t - t0), segf(sl, t - t0), s);
                 cur = segf(sl, t - t0);
             }
         }
@@ -811,6 +845,10 @@ lbm_status lbm_create(const lbm_params *p, lbm_ctx **out) {
     if ((e = dev_alloc(&c->q, (size_t)c->n * sizeof(double))) != cudaSuccess) return bail(e, "cudaMalloc(q)");
     c->fused = p->prec == LBM_F32 && !(p->flags & LBM_FLAG_TWO_PASS) &&
                fused_step_supported(model_of<float>(c), p->grad == LBM_GRAD_CDM, radius);
+    c->wide = !c->fused && (p->prec == LBM_F64 || !(p->flags & LBM_FLAG_F32_ARITH)) && wide_step_supported(*p);
+    if (c->wide && p->grad == LBM_GRAD_HDM &&
+        (e = dev_alloc(&c->sums, wide_sums_bytes(p->nx, p->ny))) != cudaSuccess)
+        return bail(e, "cudaMalloc(block sums)");
     if (c->fused) {
         size_t qb = sizeof(float) * (size_t)fused_q_pitch(p->nx) * p->ny;
         if ((e = dev_alloc(&c->qpad[0], qb)) != cudaSuccess) return bail(e, "cudaMalloc(qpad0)");
@@ -1161,18 +1199,16 @@ lbm_status lbm_step(lbm_ctx *c, int nsteps) {
     lbm_status st = check_ready(c);
     if (st != LBM_OK) return st;
     if (nsteps < 0) return fail(c, LBM_E_INVALID, "nsteps must be >= 0");
-    if (is_f64(c)) {
-        Model<double> m = model_of<double>(c);
-        for (int s = 0; s < nsteps; ++s) CK(c, step_once<double>(c, m), "step");
-    } else if (c->fused) {
+    if (c->fused) {
         Model<float> m = model_of<float>(c);
         for (int s = 0; s < nsteps; ++s) CK(c, step_fused(c, m), "fused step");
-    } else if (c->p.flags & LBM_FLAG_F32_ARITH) {
+    } else if (!is_f64(c) && (c->p.flags & LBM_FLAG_F32_ARITH)) {
         Model<float> m = model_of<float>(c);
-        for (int s = 0; s < nsteps; ++s) CK(c, step_once<float>(c, m), "step");
+        for (int s = 0; s < nsteps; ++s) CK(c, step_once_f32(c, m), "step");
     } else {
         Model<double> m = model_of<double>(c);
-        for (int s = 0; s < nsteps; ++s) CK(c, step_once_mixed(c, m), "step");
+        for (int s = 0; s < nsteps; ++s)
+            CK(c, is_f64(c) ? step_once_wide<double>(c, m) : step_once_wide<float>(c, m), "step");
     }
     return LBM_OK;
 }
@@ -1315,6 +1351,7 @@ void lbm_destroy(lbm_ctx *c) {
     dev_free(c->f[0]);
     dev_free(c->f[1]);
     dev_free(c->q);
+    dev_free(c->sums);
     dev_free(c->qpad[0]);
     dev_free(c->qpad[1]);
     dev_free(c->mom);

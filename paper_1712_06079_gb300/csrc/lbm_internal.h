@@ -86,6 +86,22 @@ cudaError_t launch_collide_mixed(const Model<double> &m, bool sc, bool cdm, cons
 cudaError_t launch_moments_mixed(const Model<double> &m, bool sc, bool cdm, const float *f, const double *q,
                                  float *rho, float *vx, float *vy, cudaStream_t s);
 
+// The same two passes in FP64 arithmetic with the HDM by block sums
+// (wide_step.cu): TS is the storage type of f and of the outputs, q (nx ny
+// values) the potential field and sums (wide_sums_bytes) the block sums that
+// pass 1 writes and pass 2 of the same state reads (unused by the CDM).
+bool wide_step_supported(const lbm_params &p);
+size_t wide_sums_bytes(int nx, int ny);
+template <typename TS>
+cudaError_t launch_wide_potential(const Model<double> &m, bool sc, bool cdm, const TS *f, double *q, double *sums,
+                                  int *err, cudaStream_t s);
+template <typename TS>
+cudaError_t launch_wide_collide(const Model<double> &m, bool sc, bool cdm, const TS *f, const double *q,
+                                double *sums, TS *fout, cudaStream_t s);
+template <typename TS>
+cudaError_t launch_wide_moments(const Model<double> &m, bool sc, bool cdm, const TS *f, const double *q, double *sums,
+                                TS *rho, TS *vx, TS *vy, cudaStream_t s);
+
 // HDM (Eq. 20) or CDM (Eq. 15 times 1/c_s^2) gradient of the periodic field
 // q (nx * ny, row-major) on a grid of spacing h into gx, gy.
 template <typename T>

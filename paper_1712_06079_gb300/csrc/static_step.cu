@@ -20,34 +20,46 @@ namespace {
 
 static __device__ __align__(256) unsigned char g_static_scratch[LBM_STATIC_SCRATCH_BYTES];
 
+// Block sums of the potential field (wide_step.cu); a lattice whose sums do not
+// fit (under 4 cells one way and close to the size limit) takes the direct
+// stencil instead.
+constexpr size_t kSumsBytes = 3u << 20;
+static __device__ __align__(256) unsigned char g_static_sums[kSumsBytes];
+
 constexpr int kMaxDevices = 64;
 constexpr size_t kErrBytes = 256;  // error word, padded so the field stays 256-byte aligned
 
 std::mutex g_scratch_mutex;
-void *g_scratch_ptr[kMaxDevices] = {};
+void *g_scratch_ptr[kMaxDevices] = {}, *g_sums_ptr[kMaxDevices] = {};
 
-// Device address of the scratch array on the current device.  The array's
+// Device addresses of the scratch arrays on the current device.  An array's
 // name is a host-side stand-in in host code, so its address is looked up
 // once per device with that device current.
-lbm_status scratch_on_current_device(void **out) {
+lbm_status scratch_on_current_device(void **out, void **sums) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return LBM_E_CUDA;
     std::lock_guard<std::mutex> lock(g_scratch_mutex);
     if (!g_scratch_ptr[dev]) {
         void *p = nullptr;
         if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) return LBM_E_CUDA;
+        void *ps = nullptr;
+        if (cudaGetSymbolAddress(&ps, g_static_sums) != cudaSuccess || !ps) return LBM_E_CUDA;
         g_scratch_ptr[dev] = p;
+        g_sums_ptr[dev] = ps;
     }
     *out = g_scratch_ptr[dev];
+    *sums = g_sums_ptr[dev];
     return LBM_OK;
 }
 
-// The step of lbm_step's two-pass form: T is the arithmetic type, TS the
-// storage type of f (FP32 lattices: FP32 distributions, FP64 arithmetic and an
-// FP64 potential field, as lbm_step computes them).
-template <typename TS, typename T>
-lbm_status run_step(const lbm_params &p, const lbm::ModelScalars &ms, const void *f_in, void *f_out, void *scratch) {
+// The step of lbm_step's two-pass form in FP64 arithmetic; TS is the storage
+// type of f (FP32 lattices: FP32 distributions and an FP64 potential field, as
+// lbm_step computes them).
+template <typename TS>
+lbm_status run_step(const lbm_params &p, const lbm::ModelScalars &ms, const void *f_in, void *f_out, void *scratch,
+                    void *sums) {
     using namespace lbm;
+    using T = double;
     Model<T> m{};
     m.nx = p.nx;
     m.ny = p.ny;
@@ -75,7 +87,11 @@ lbm_status run_step(const lbm_params &p, const lbm::ModelScalars &ms, const void
     const bool sc = p.force == LBM_FORCE_SC, cdm = p.grad == LBM_GRAD_CDM;
     if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) return LBM_E_CUDA;
     cudaError_t e;
-    if constexpr (sizeof(TS) == sizeof(T)) {
+    if (wide_step_supported(p) && (cdm || wide_sums_bytes(p.nx, p.ny) <= kSumsBytes)) {
+        e = launch_wide_potential<TS>(m, sc, cdm, (const TS *)f_in, q, (double *)sums, err, s);
+        if (e == cudaSuccess)
+            e = launch_wide_collide<TS>(m, sc, cdm, (const TS *)f_in, q, (double *)sums, (TS *)f_out, s);
+    } else if constexpr (sizeof(TS) == sizeof(T)) {
         e = launch_potential<T>(m, sc, (const T *)f_in, q, err, s);
         if (e == cudaSuccess) e = launch_collide<T>(m, sc, cdm, (const T *)f_in, q, (T *)f_out, s);
     } else {
@@ -103,9 +119,9 @@ extern "C" lbm_status lbm_step_noalloc(const lbm_params *p, const void *f_in, vo
     if ((long long)p->nx * p->ny > max_cells()) return LBM_E_INVALID;
     lbm::ModelScalars ms;
     if (lbm::model_scalars(*p, &ms) != LBM_OK) return LBM_E_INVALID;
-    void *scratch = nullptr;
-    lbm_status st = scratch_on_current_device(&scratch);
+    void *scratch = nullptr, *sums = nullptr;
+    lbm_status st = scratch_on_current_device(&scratch, &sums);
     if (st != LBM_OK) return st;
-    return p->prec == LBM_F64 ? run_step<double, double>(*p, ms, f_in, f_out, scratch)
-                              : run_step<float, double>(*p, ms, f_in, f_out, scratch);
+    return p->prec == LBM_F64 ? run_step<double>(*p, ms, f_in, f_out, scratch, sums)
+                              : run_step<float>(*p, ms, f_in, f_out, scratch, sums);
 }

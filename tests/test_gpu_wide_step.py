@@ -1,0 +1,75 @@
+"""The FP64-arithmetic two-pass step with the HDM by block sums (wide_step.cu)
+against the oracle, whose operator is the cyclic tridiagonal solve: lines
+shorter and longer than a block of 8 cells and than the 40 cells that are
+joined, ends in a block of every length, mirrored columns between walls."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1712_06079_gb300 import inputs, lbm
+
+pytestmark = pytest.mark.gpu
+
+
+def make(nx, ny, prec, force="sc", grad="hdm", tau=1.0, walls=False, radius=0):
+    t = inputs.EOS_TABLE["cs"]
+    gp = lbm.Params(nx=nx, ny=ny, eos="cs", a=t["a"], b=t["b"], Tr=0.8, k=t["k"], tau=tau, force=force, grad=grad,
+                    prec=prec, walls=walls, hdm_radius=radius, two_pass=True)
+    op = oracle.params_at(nx, ny, "cs", t["a"], t["b"], 0.8, k=t["k"], tau=tau, force=force, grad=grad, walls=walls)
+    g, l, _ = oracle.maxwell(op)
+    xi = inputs.uniform01(nx * 131 + ny, 12 * nx * ny).reshape(12, ny, nx)
+    f = oracle.init(op, g + (l - g) * xi[11], 0.1 * (xi[0] - 0.5), 0.1 * (xi[1] - 0.5))
+    return gp, op, f * (1.0 + 1e-3 * (xi[2:11] - 0.5))
+
+
+SIZES = [(2, 2), (3, 9), (7, 40), (8, 8), (9, 17), (16, 5), (15, 41), (39, 81), (23, 64), (121, 10), (130, 133)]
+
+
+@pytest.mark.parametrize("nx,ny", SIZES)
+@pytest.mark.parametrize("force,grad,tau,walls", [("sc", "hdm", 1.0, False), ("zc", "hdm", 0.8, False),
+                                                  ("sc", "hdm", 1.2, True), ("zc", "hdm", 1.0, True),
+                                                  ("sc", "cdm", 0.9, True), ("zc", "cdm", 1.0, False)])
+def test_one_step_is_the_oracles(nx, ny, force, grad, tau, walls):
+    # FP64: the per-step bar of 1e-12 on every population (a random density
+    # field, so the derivative is as rough as the lattice carries)
+    gp, op, f0 = make(nx, ny, "f64", force, grad, tau, walls)
+    with lbm.Lattice(gp) as lat:
+        lat.set_f(f0)
+        r, vx, vy = lat.moments()   # (of the given state: a step of so rough a field may leave the stable range)
+        lat.step(1)
+        fg = lat.get_f()
+    fo = oracle.step(op, f0)
+    scale = np.abs(fo).max(axis=0)   # (a small population of a cell can cancel: relative to the cell's largest)
+    assert np.max(np.abs(fg - fo) / scale) < 1e-12
+    ro, vxo, vyo = oracle.moments(op, f0)
+    assert np.max(np.abs(r / ro - 1)) < 1e-12
+    assert max(np.abs(vx - vxo).max(), np.abs(vy - vyo).max()) < 1e-12 * max(1.0, np.abs(vxo).max())
+
+
+@pytest.mark.parametrize("nx,ny", [(9, 17), (39, 81), (130, 133)])
+def test_fp32_storage_adds_one_rounding(nx, ny):
+    # FP32 distributions, FP64 arithmetic: the oracle's step of the stored
+    # state, rounded once (half an ulp, 6e-8 relative to each population)
+    gp, op, f0 = make(nx, ny, "f32")
+    f0 = f0.astype(np.float32).astype(np.float64)
+    with lbm.Lattice(gp) as lat:
+        lat.set_f(f0)
+        lat.step(1)
+        fg = lat.get_f()
+    fo = oracle.step(op, f0)
+    assert np.max(np.abs(fg - fo) / np.abs(fo).max(axis=0)) < 6.0e-8
+
+
+def test_a_requested_radius_keeps_its_truncation():
+    # hdm_radius is part of the result: 8 and the automatic radius differ by
+    # about r^9 = 2e-4 of the derivative on a rough field, and 40 equals it
+    out = {}
+    for radius in (0, 8, 40):
+        gp, op, f0 = make(64, 48, "f64", radius=radius)
+        with lbm.Lattice(gp) as lat:
+            lat.set_f(f0)
+            lat.step(1)
+            out[radius] = lat.get_f()
+    scale = np.abs(out[0]).max()
+    assert np.abs(out[40] - out[0]).max() < 1e-14 * scale * 100
+    assert np.abs(out[8] - out[0]).max() > 1e-9 * scale
