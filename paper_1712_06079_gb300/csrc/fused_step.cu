@@ -75,6 +75,11 @@
 // steps, never for walls or the CDM) also writes, for every cell of its own rows, the
 // record of f(t) the adjoint step reads in place of f(t) and the stencil
 // field: rho and j (Eq. 3) and the two HDM derivatives, five planes of nx ny.
+//
+// The MOM variant sweeps the state the same way but, instead of colliding,
+// writes rho (Eq. 3) and the half-step velocity of Eq. 11: 40 B in and 12 B out
+// per cell from the field the last step left, where the two-pass kernels'
+// moments read f twice and differentiate cell by cell.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -120,6 +125,8 @@ struct FusedArgs {
     const float *qin;   // padded field of f(t): row pitch qpitch, column x at x + QG
     float *qout;        // padded field of f(t+1)
     float *rec;         // TAPE: record of f(t), planes rho, jx, jy, Dx, Dy (nx ny each)
+    float *mom[3];      // MOM: rho, vx, vy (nx ny each)
+    int mom4;           // MOM: the three arrays are 16-byte aligned
     int *err;
     int qpitch;         // nx + 2 * QG
     int seg_h;          // rows per CTA segment
@@ -257,10 +264,11 @@ __device__ __forceinline__ bool range_ok(long long off, long long len, long long
     return in_bounds(off, n - len + 1, err);
 }
 
-template <bool SC, bool TAU1, int EOS, bool WALLS, bool TAPE = false, bool CDMG = false>
+template <bool SC, bool TAU1, int EOS, bool WALLS, bool TAPE = false, bool CDMG = false, bool MOM = false>
 __global__ void __launch_bounds__(NTHR, 2) fused_step_kernel(const __grid_constant__ FusedArgs A) {
     static_assert(!(TAPE && WALLS), "the reverse mode takes periodic lattices");
     static_assert(!(TAPE && CDMG), "the reverse mode of CDM lattices takes the two-pass kernels");
+    static_assert(!MOM || (TAU1 && !TAPE), "the moments variant uses f(t) only for its moments");
     extern __shared__ __align__(128) unsigned char smem[];
     float *qn = reinterpret_cast<float *>(smem);               // [QRING][NW]
     float *qw = reinterpret_cast<float *>(smem + kOffQw);      // [2][SLAB][WW]
@@ -546,18 +554,8 @@ __global__ void __launch_bounds__(NTHR, 2) fused_step_kernel(const __grid_consta
                     }
                 }
             }
-            // force and the two velocities of the forcing (Eq. 10, 22 / 7)
-            float2 ux[2], uy[2], vx[2], vy[2], au[2], av[2], moved[2];
-            {   // the 4 densities positive and finite: the least above 0, the sum finite (a NaN or
-                // an infinity makes it not; a sum past the FP32 range flags a blown-up state too)
-                const float2 rs = add2(r2[0], r2[1]);
-                const float rmin = fminf(fminf(r2[0].x, r2[0].y), fminf(r2[1].x, r2[1].y));
-                unstable |= active && !(rmin > 0.f && rs.x + rs.y < INFINITY);
-            }
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            auto force2 = [&](int h, float2 &Fx, float2 &Fy) {   // the interaction force on cells 2h, 2h + 1
                 const float2 gx = make_float2(dx[2 * h], dx[2 * h + 1]), gy = make_float2(dy[2 * h], dy[2 * h + 1]);
-                float2 Fx, Fy;
                 if (SC) {   // Eq. 22: F = -2 s Phi grad Phi, s Phi the stored field at the cell
                     const float2 m2q = mul2(splat2(-2.0f), make_float2(qc[2 * h], qc[2 * h + 1]));
                     Fx = mul2(m2q, gx);
@@ -566,6 +564,47 @@ __global__ void __launch_bounds__(NTHR, 2) fused_step_kernel(const __grid_consta
                     Fx = mul2(splat2(-1.0f), gx);
                     Fy = mul2(splat2(-1.0f), gy);
                 }
+            };
+            {   // the 4 densities positive and finite: the least above 0, the sum finite (a NaN or
+                // an infinity makes it not; a sum past the FP32 range flags a blown-up state too)
+                const float2 rs = add2(r2[0], r2[1]);
+                const float rmin = fminf(fminf(r2[0].x, r2[0].y), fminf(r2[1].x, r2[1].y));
+                unstable |= active && !(rmin > 0.f && rs.x + rs.y < INFINITY);
+            }
+            if constexpr (MOM) {   // rho and v = (j + F/2) / rho (Eq. 11) of the lane's 4 cells of an own row
+                if (interior && yc >= ys && yc < ys + hseg) {
+                    float2 v2[2], w2[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        float2 Fx, Fy;
+                        force2(h, Fx, Fy);
+                        const float2 inv = make_float2(__fdividef(1.0f, r2[h].x), __fdividef(1.0f, r2[h].y));
+                        v2[h] = mul2(fma2(splat2(0.5f), Fx, jx2[h]), inv);
+                        w2[h] = mul2(fma2(splat2(0.5f), Fy, jy2[h]), inv);
+                    }
+                    const long long o = (long long)yc * nx + xg;
+                    auto put = [&](float *p, const float2 (&v)[2]) {
+                        if (!range_ok(o, 4, 4LL * A.n4, A.err)) return;
+                        if (A.mom4) {
+                            *reinterpret_cast<float4 *>(p + o) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+                        } else {
+                            p[o] = v[0].x;
+                            p[o + 1] = v[0].y;
+                            p[o + 2] = v[1].x;
+                            p[o + 3] = v[1].y;
+                        }
+                    };
+                    put(A.mom[0], r2);
+                    put(A.mom[1], v2);
+                    put(A.mom[2], w2);
+                }
+            } else {
+            // force and the two velocities of the forcing (Eq. 10, 22 / 7)
+            float2 ux[2], uy[2], vx[2], vy[2], au[2], av[2], moved[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float2 Fx, Fy;
+                force2(h, Fx, Fy);
                 const float2 inv = make_float2(__fdividef(1.0f, r2[h].x), __fdividef(1.0f, r2[h].y));
                 ux[h] = mul2(jx2[h], inv);
                 uy[h] = mul2(jy2[h], inv);
@@ -671,6 +710,7 @@ __global__ void __launch_bounds__(NTHR, 2) fused_step_kernel(const __grid_consta
                 const int slot = (rd0 + k - 1) % PROWS;
                 *reinterpret_cast<float4 *>(ps + (k * PROWS + slot) * NW + 4 * lane) = part[k];
             }
+            }
         }
         if (s + 1 < nslab) {   // slab s + 1's recurrences: its last ring chunk, then the column phase
             const int c = s + 1 + QAHEAD;
@@ -682,6 +722,7 @@ __global__ void __launch_bounds__(NTHR, 2) fused_step_kernel(const __grid_consta
             break;
         }
 
+        if constexpr (MOM) continue;
         // ---- rho(t+1) and the potential of row yo = ys + 8s - 2 + warp ----
         const int yo = ys + SLAB * s - 2 + warp;
         if (interior && yo >= ys && yo < ys + hseg) {
@@ -769,25 +810,18 @@ cudaError_t launch_potential_padded(const Model<float> &m, bool sc, const float 
     return cudaGetLastError();
 }
 
-cudaError_t launch_fused_step(const Model<float> &m, bool sc, bool cdm, const float *f, const float *qin,
-                              float *fout, float *qout, int *err, int seg_rows, cudaStream_t s, bool pdl, float *rec,
-                              bool rev) {
-    if (rec && (m.walls || cdm)) return cudaErrorInvalidValue;
-    FusedArgs a;
+namespace {
+
+FusedArgs fused_args(const Model<float> &m, const float *f, const float *qin, int *err, int seg_rows, bool rev) {
+    FusedArgs a{};
     a.m = m;
     a.f = f;
-    a.fout = fout;
     a.qin = qin;
-    a.qout = qout;
-    a.rec = rec;
     a.err = err;
     a.qpitch = fused_q_pitch(m.nx);
     a.seg_h = seg_rows;
     a.n4 = (int)((long long)m.nx * m.ny / 4);
     a.rev = rev ? 1 : 0;
-    if (seg_rows < 1) return cudaErrorInvalidValue;
-    dim3 grid((m.nx + TXI - 1) / TXI, (m.ny + seg_rows - 1) / seg_rows);
-    if (grid.y > 65535) return cudaErrorInvalidValue;
     a.w1y = m.wy[1];
     a.w2y = m.wy[2];
     const double r = 0.5 * (std::sqrt(5.0) - 3.0);   // root of r^2/3 + r + 1/3 = 0 (Eq. 20's operator)
@@ -797,6 +831,59 @@ cudaError_t launch_fused_step(const Model<float> &m, bool sc, bool cdm, const fl
     a.ry5 = (float)std::pow(r, 5);
     a.ry12 = (float)std::pow(r, 12);
     a.ry25 = (float)std::pow(r, 25);
+    return a;
+}
+
+cudaError_t launch_sweep(void (*kern)(const FusedArgs), const FusedArgs &a, cudaStream_t s, bool pdl) {
+    if (a.seg_h < 1) return cudaErrorInvalidValue;
+    const dim3 grid((a.m.nx + TXI - 1) / TXI, (a.m.ny + a.seg_h - 1) / a.seg_h);
+    if (grid.y > 65535) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(NTHR);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    e = cudaLaunchKernelEx(&cfg, kern, a);
+    if (e != cudaSuccess) return e;
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_fused_moments(const Model<float> &m, bool sc, bool cdm, const float *f, const float *qin, float *rho,
+                                 float *vx, float *vy, int *err, int seg_rows, cudaStream_t s, bool rev) {
+    FusedArgs a = fused_args(m, f, qin, err, seg_rows, rev);
+    a.mom[0] = rho;
+    a.mom[1] = vx;
+    a.mom[2] = vy;
+    // (the caller's arrays may start at any element: 16-byte stores only where all three are aligned)
+    a.mom4 = ((reinterpret_cast<uintptr_t>(rho) | reinterpret_cast<uintptr_t>(vx) | reinterpret_cast<uintptr_t>(vy)) & 15) == 0;
+    // the equation of state enters only through the stored field: one variant for all
+#define LBM_MOM(SC, W, C) fused_step_kernel<SC, true, LBM_EOS_CS, W, false, C, true>
+    void (*kern)(const FusedArgs) =
+        cdm ? (m.walls ? (sc ? LBM_MOM(true, true, true) : LBM_MOM(false, true, true))
+                       : (sc ? LBM_MOM(true, false, true) : LBM_MOM(false, false, true)))
+            : (m.walls ? (sc ? LBM_MOM(true, true, false) : LBM_MOM(false, true, false))
+                       : (sc ? LBM_MOM(true, false, false) : LBM_MOM(false, false, false)));
+#undef LBM_MOM
+    return launch_sweep(kern, a, s, true);
+}
+
+cudaError_t launch_fused_step(const Model<float> &m, bool sc, bool cdm, const float *f, const float *qin,
+                              float *fout, float *qout, int *err, int seg_rows, cudaStream_t s, bool pdl, float *rec,
+                              bool rev) {
+    if (rec && (m.walls || cdm)) return cudaErrorInvalidValue;
+    FusedArgs a = fused_args(m, f, qin, err, seg_rows, rev);
+    a.fout = fout;
+    a.qout = qout;
+    a.rec = rec;
     const bool tau1 = m.omega == 1.0f;
     void (*kern)(const FusedArgs) = nullptr;
 #define LBM_PICK(E)                                                                                        \
@@ -830,21 +917,7 @@ cudaError_t launch_fused_step(const Model<float> &m, bool sc, bool cdm, const fl
     default: LBM_PICK(LBM_EOS_RKS); break;
     }
 #undef LBM_PICK
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(NTHR);
-    cfg.dynamicSmemBytes = kSmemBytes;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    e = cudaLaunchKernelEx(&cfg, kern, a);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    return launch_sweep(kern, a, s, pdl);
 }
 
 }  // namespace lbm

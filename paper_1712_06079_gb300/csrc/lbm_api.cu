@@ -343,7 +343,27 @@ template <typename TS>
 cudaError_t moments_into(lbm_ctx *c, TS *r, TS *vx, TS *vy) {
     const TS *f = (const TS *)c->f[c->cur];
     if constexpr (std::is_same_v<TS, float>) {
-        if (c->fused || (c->p.flags & LBM_FLAG_F32_ARITH)) {
+        if (c->fused) {
+            // from the field the last step left; before the first step (and under
+            // capture, where a replay may meet another state) the field is formed
+            // from f, into the two-pass field's memory: 8 nx ny bytes hold the
+            // 4 (nx + 64) ny of the padded layout, as nx >= 64 here
+            Model<float> mf = model_of<float>(c);
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {   // (an unusable stream: the launch says so)
+                cudaGetLastError();
+                cap = cudaStreamCaptureStatusActive;
+            }
+            const float *q = (const float *)c->qpad[c->cur];
+            if (!c->qpad_valid || cap != cudaStreamCaptureStatusNone) {
+                const cudaError_t e = launch_potential_padded(mf, is_sc(c), f, (float *)c->q, c->err, c->stream);
+                if (e != cudaSuccess) return e;
+                q = (const float *)c->q;
+            }
+            return launch_fused_moments(mf, is_sc(c), is_cdm(c), f, q, r, vx, vy, c->err, seg_rows_of(c), c->stream,
+                                        c->fused_rev);
+        }
+        if (c->p.flags & LBM_FLAG_F32_ARITH) {
             Model<float> mf = model_of<float>(c);
             cudaError_t e = launch_potential<float>(mf, is_sc(c), f, (float *)c->q, c->err, c->stream);
             if (e != cudaSuccess) return e;

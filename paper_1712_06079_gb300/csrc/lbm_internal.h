@@ -136,6 +136,12 @@ cudaError_t launch_fused_step(const Model<float> &m, bool sc, bool cdm, const fl
                               float *fout, float *qout, int *err, int seg_rows, cudaStream_t s, bool pdl = true,
                               float *rec = nullptr, bool rev = false);
 
+// rho (Eq. 3) and the half-step velocity (Eq. 11) of state f with its padded
+// potential qin, by the same sweep; rho, vx, vy: nx ny floats each, of any
+// alignment.
+cudaError_t launch_fused_moments(const Model<float> &m, bool sc, bool cdm, const float *f, const float *qin, float *rho,
+                                 float *vx, float *vy, int *err, int seg_rows, cudaStream_t s, bool rev);
+
 // Adjoint (reverse-time) step (adjoint.cu): from lambda = dL/df at t+1 and the
 // state f at t with its stencil field q (row y, column x at
 // q[y * qpitch + qoff + x]; |q| = Phi for the Shan-Chen form, U for
