@@ -297,17 +297,16 @@ __global__ void obs_partial_kernel(long long n, const T *__restrict__ rho, const
         for (int k = 0; k < 6; ++k) partial[k * gridDim.x + blockIdx.x] = sh[k][0];
 }
 
+// The blocks' partials of one quantity per warp (six warps), lane by lane and
+// then by shuffles in a fixed order, so the sums are reproducible.
 __global__ void obs_final_kernel(int nb, const double *__restrict__ partial, lbm_obs *out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double s[6] = {0, 0, 0, 0, INFINITY, -INFINITY};
-    for (int b = 0; b < nb; ++b) {
-        s[0] += partial[b]; s[1] += partial[nb + b]; s[2] += partial[2 * nb + b];
-        s[3] = fmax(s[3], partial[3 * nb + b]);
-        s[4] = fmin(s[4], partial[4 * nb + b]);
-        s[5] = fmax(s[5], partial[5 * nb + b]);
-    }
-    out->mass = s[0]; out->mom_x = s[1]; out->mom_y = s[2];
-    out->max_speed = s[3]; out->rho_min = s[4]; out->rho_max = s[5];
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double s = k < 4 ? 0.0 : (k == 4 ? INFINITY : -INFINITY);
+    auto join = [&](double a, double b) { return k < 3 ? a + b : (k == 4 ? fmin(a, b) : fmax(a, b)); };
+    for (int b = lane; b < nb; b += 32) s = join(s, partial[k * nb + b]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s = join(s, __shfl_down_sync(0xffffffffu, s, o));
+    if (lane == 0) (&out->mass)[k] = s;   // mass, mom_x, mom_y, max_speed, rho_min, rho_max: six doubles in a row
 }
 
 }  // namespace
@@ -417,7 +416,7 @@ template <typename T>
 cudaError_t launch_observables(long long n, const T *rho, const T *vx, const T *vy, double *partial, lbm_obs *out,
                                cudaStream_t s) {
     obs_partial_kernel<T><<<kObsBlocks, kObsThreads, 0, s>>>(n, rho, vx, vy, partial);
-    obs_final_kernel<<<1, 32, 0, s>>>(kObsBlocks, partial, out);
+    obs_final_kernel<<<1, 192, 0, s>>>(kObsBlocks, partial, out);
     return cudaGetLastError();
 }
 
