@@ -789,16 +789,42 @@ bool fused_step_supported(const Model<float> &m, bool cdm, int radius) {
 int fused_q_pitch(int nx) { return nx + 2 * QG; }
 
 // A segment of h rows collides 8 ceil((h + 2) / 8) rows (its own, the one above
-// and the one below, in whole slabs) and stages h + 66 potential rows for
-// d/dy, so h = 8k - 2 wastes no collided rows.  The tallest such segment that
-// still gives every SM a CTA keeps the halo overhead lowest (measured on 512^2
-// to 4096^2 lattices: 14, 62, 126, 126 rows); smaller grids leave SMs idle.
-int fused_auto_seg_rows(int nx, int ny, int num_sms) {
-    const long long strips = (nx + TXI - 1) / TXI;
-    const int cand[] = {126, 62, 30, 14, 6};
-    for (int h : cand)
-        if (strips * ((ny + h - 1) / h) >= num_sms) return h;
-    return 6;
+// and the one below, in whole slabs), so h = 8k - 2 wastes no collided rows.  Two
+// CTAs share an SM, and a CTA's time is its number of slabs (about 3.5 us each,
+// whether or not it shares the SM), so a launch takes waves x slabs: for each
+// number of waves the shortest segments that fit into it are candidates, and the
+// fewest wave-slabs win, ties to fewer waves.  us per step at the height
+// this picks, with the tallest of 126, 62, 30, 14, 6 rows that gives every SM a CTA
+// (the rule before), and at the best of all heights: 768^2 12.0, 15.0, 12.0; 1024^2
+// 18.0, 26.1, 18.0; 1536^2 32.6, 51.1, 32.6; 2048^2 57.7, 61.4, 57.3; 3072^2 129, 148,
+// 126; 4096^2 225, 227, 221 (tau 0.9: 225, 240, 225).  The CDM variant has no column
+// recurrences to start, so short segments cost it little and on large lattices the
+// memory system's tail decides instead: it follows this rule while one wave of at
+// most 9 slabs does (1024^2 19.1 -> 13.5 us), else the one before (2048^2 57.6 us
+// against 58.5 at one wave of 17 slabs).
+int fused_auto_seg_rows(int nx, int ny, int num_sms, bool cdm) {
+    const long long strips = (nx + TXI - 1) / TXI, slots = 2LL * num_sms;
+    // slabs of the shortest segments that make at most `waves` full waves (0: none do)
+    auto slabs_for = [&](int waves) -> long long {
+        const long long segs = slots * waves / strips;   // segments a strip may have
+        if (segs < 1) return 0;
+        return ((ny + segs - 1) / segs + 2 + SLAB - 1) / SLAB;
+    };
+    if (cdm && !(slabs_for(1) >= 1 && slabs_for(1) <= 9)) {
+        const int cand[] = {126, 62, 30, 14, 6};
+        for (int h : cand)
+            if (strips * ((ny + h - 1) / h) >= num_sms) return h;
+        return 6;
+    }
+    long long best = 0, rows = 126;   // (strips alone beyond the waves tried: tall segments)
+    for (int w = 1; w <= (cdm ? 1 : 8); ++w) {
+        const long long k = slabs_for(w);
+        if (k >= 1 && (best == 0 || w * k < best)) {
+            best = w * k;
+            rows = SLAB * k - 2;
+        }
+    }
+    return (int)rows;
 }
 
 cudaError_t launch_potential_padded(const Model<float> &m, bool sc, const float *f, float *qpad, int *err,

@@ -310,7 +310,7 @@ cudaError_t step_once_f32(lbm_ctx *c, const Model<float> &m) {
 }
 
 int seg_rows_of(const lbm_ctx *c) {
-    return c->seg_rows > 0 ? c->seg_rows : fused_auto_seg_rows(c->p.nx, c->p.ny, c->num_sms);
+    return c->seg_rows > 0 ? c->seg_rows : fused_auto_seg_rows(c->p.nx, c->p.ny, c->num_sms, is_cdm(c));
 }
 
 // One time step by the single-pass FP32 kernel.

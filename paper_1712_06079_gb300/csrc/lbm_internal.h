@@ -122,7 +122,7 @@ cudaError_t launch_observables(long long n, const T *rho, const T *vx, const T *
 // the segment height for a lattice on a GPU with num_sms SMs.
 bool fused_step_supported(const Model<float> &m, bool cdm, int radius);
 int fused_q_pitch(int nx);
-int fused_auto_seg_rows(int nx, int ny, int num_sms);
+int fused_auto_seg_rows(int nx, int ny, int num_sms, bool cdm);
 cudaError_t launch_potential_padded(const Model<float> &m, bool sc, const float *f, float *qpad, int *err,
                                     cudaStream_t s);
 // pdl: launch with programmatic serialization (the grid may be scheduled while
