@@ -855,13 +855,21 @@ __global__ void adj_initial_kernel(int nx, int ny, int nlam, const T *lam, long 
     }
 }
 
-// Sum of the slots in a fixed order (lane k takes slots k, k + 32, ... in
-// turn, then a fixed shuffle tree): one warp, reproducible.
-__global__ void sum_slots_kernel(const double *slots, int nslots, double *out) {
+// Sum of the slots in a fixed order (thread k takes slots k, k + 1024, ... in
+// turn, then fixed shuffle trees): one block, reproducible.
+__global__ void __launch_bounds__(1024) sum_slots_kernel(const double *slots, int nslots, double *out) {
+    __shared__ double part[32];
     double s = 0.0;
-    for (int i = threadIdx.x; i < nslots; i += 32) s += slots[i];
+    for (int i = threadIdx.x; i < nslots; i += 1024) s += slots[i];
+    for (int half = 0; half < 2; ++half) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (half == 0) {
+            if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+            __syncthreads();
+            s = part[threadIdx.x & 31];
+        }
+    }
     if (threadIdx.x == 0) *out = s;
 }
 
@@ -1058,7 +1066,7 @@ cudaError_t launch_adjoint_initial(int nx, int ny, const AdjLayout &l, const T *
 }
 
 cudaError_t launch_sum_slots(const double *slots, int nslots, double *out, cudaStream_t s) {
-    sum_slots_kernel<<<1, 32, 0, s>>>(slots, nslots, out);
+    sum_slots_kernel<<<1, 1024, 0, s>>>(slots, nslots, out);
     return cudaGetLastError();
 }
 

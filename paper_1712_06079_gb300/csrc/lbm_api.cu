@@ -157,6 +157,7 @@ struct lbm_ctx {
     cudaEvent_t rec_done[kTapeSlots] = {}, adj_done[kTapeSlots] = {}, bw_start = nullptr;
     void *lam[2] = {nullptr, nullptr};
     void *aux = nullptr;
+    double *asums = nullptr;          // block sums of D_bar (FP64 block-sum lattices)
     double *slots = nullptr;
 };
 
@@ -214,6 +215,10 @@ bool is_cdm(const lbm_ctx *c) { return c->p.grad == LBM_GRAD_CDM; }
 // the padded layout) for HDM lattices only; CDM lattices tape with the
 // two-pass kernels.
 bool tape_fused(const lbm_ctx *c) { return c->fused && !is_cdm(c); }
+// FP64 lattices on the block-sum step (wide_step.cu) tape its record of every
+// state, as the single-pass lattices tape theirs.
+bool tape_wide(const lbm_ctx *c) { return c->wide && is_f64(c); }
+bool tape_rec(const lbm_ctx *c) { return tape_fused(c) || tape_wide(c); }
 
 cudaError_t take_event(lbm_ctx *c, cudaEvent_t *ev) {
     if (!c->event_pool.empty()) {
@@ -473,8 +478,10 @@ void free_tape(lbm_ctx *c) {
     c->rstream = c->astream = nullptr;
     c->bw_start = nullptr;
     dev_free(c->aux);
+    dev_free(c->asums);
     dev_free(c->slots);
     c->aux = nullptr;
+    c->asums = nullptr;
     c->slots = nullptr;
     for (int k = 0; k < 2; ++k) {
         dev_free(c->tmp[k]);
@@ -494,28 +501,39 @@ cudaError_t tape_potential(lbm_ctx *c, const Model<T> &m, const void *f, void *q
     else return launch_potential<T>(m, is_sc(c), (const T *)f, (T *)q, c->err, s);
 }
 template <typename T>
-cudaError_t tape_collide(lbm_ctx *c, const Model<T> &m, const void *f, const void *q, void *g, cudaStream_t s) {
-    if constexpr (std::is_same_v<T, double>)
+cudaError_t tape_collide(lbm_ctx *c, const Model<T> &m, const void *f, const void *q, void *g, void *rec,
+                         cudaStream_t s) {
+    if constexpr (std::is_same_v<T, double>) {
+        if (rec)   // (block-sum lattices)
+            return launch_wide_collide_rec(m, is_sc(c), is_cdm(c), (const double *)f, (const double *)q, c->sums,
+                                           (double *)g, (double *)rec, s);
         return wide_collide(c, m, (const double *)f, (const double *)q, (double *)g, s);
-    else return launch_collide<T>(m, is_sc(c), is_cdm(c), (const T *)f, (const T *)q, (T *)g, s);
+    } else {
+        return launch_collide<T>(m, is_sc(c), is_cdm(c), (const T *)f, (const T *)q, (T *)g, s);
+    }
 }
 
 // One forward step from state `src` to `dst` (explicit buffers).  Single-pass
 // path: qsrc holds the padded stencil field of src (valid on entry) and qdst
 // receives that of dst.  Two-pass path: the potential of src is formed into
-// qsrc first (qdst unused).  rec (single-pass): where the record of src goes,
-// or nullptr.
+// qsrc first (qdst unused).  rec: where the record of src goes, or nullptr.
 template <typename T>
 cudaError_t tape_step(lbm_ctx *c, const Model<T> &m, const void *src, void *dst, void *qsrc, void *qdst,
-                      float *rec, bool rev) {
+                      void *rec, bool rev) {
     if constexpr (std::is_same_v<T, float>) {   // (FP64 contexts never take the single-pass kernel)
         if (tape_fused(c))
             return launch_fused_step(m, is_sc(c), is_cdm(c), (const float *)src, (const float *)qsrc, (float *)dst,
-                                     (float *)qdst, c->err, seg_rows_of(c), c->stream, true, rec, rev);
+                                     (float *)qdst, c->err, seg_rows_of(c), c->stream, true, (float *)rec, rev);
     }
     cudaError_t e = tape_potential<T>(c, m, src, qsrc, c->stream);
     if (e != cudaSuccess) return e;
-    return tape_collide<T>(c, m, src, qsrc, dst, c->stream);
+    return tape_collide<T>(c, m, src, qsrc, dst, rec, c->stream);
+}
+
+// FP64 dL/dT slots of the reverse step's kernels
+template <typename T>
+int tape_slots(const lbm_ctx *c) {
+    return tape_wide(c) ? wide_adjoint_slots(c->p.nx, c->p.ny) : adjoint_slots<T>(c->p.nx, c->p.ny);
 }
 
 template <typename T>
@@ -559,12 +577,13 @@ lbm_status tape_forward(lbm_ctx *c, const T *rho0, int nsteps, int C, T *rhoT) {
             const int qpitch = tape_fused(c) ? fused_q_pitch(c->p.nx) : c->p.nx;
             const size_t qbytes = sizeof(T) * (size_t)qpitch * c->p.ny;
             const AdjLayout lay = adjoint_layout(c->p.nx, c->p.ny, tape_fused(c), tau1);
+            const int naux = lay.naux + (tape_wide(c) ? 1 : 0);   // (kappa and theta in the place of rho)
             const size_t lbytes = (size_t)lay.nlam * lay.lstride * sizeof(T);
             bool ok = true;
-            // single-pass contexts keep the forward kernel's record of every state
-            // of a segment (five planes); the others keep the states after the first
-            const size_t sbytes = tape_fused(c) ? (size_t)5 * c->n * sizeof(float) : fbytes;
-            c->seg.assign(tape_fused(c) ? kTapeSlots * C : kTapeSlots * (C > 1 ? C - 1 : 0), nullptr);
+            // contexts with a record keep it of every state of a segment (five
+            // planes); the others keep the states after the first
+            const size_t sbytes = tape_rec(c) ? (size_t)5 * c->n * sizeof(T) : fbytes;
+            c->seg.assign(tape_rec(c) ? kTapeSlots * C : kTapeSlots * (C > 1 ? C - 1 : 0), nullptr);
             c->segq.assign(kTapeSlots * C, nullptr);
             for (auto &p : c->seg) ok = ok && dev_alloc(&p, sbytes) == cudaSuccess;
             for (auto &p : c->segq) ok = ok && dev_alloc(&p, qbytes) == cudaSuccess;
@@ -576,8 +595,10 @@ lbm_status tape_forward(lbm_ctx *c, const T *rho0, int nsteps, int C, T *rhoT) {
                 ok = ok && cudaEventCreateWithFlags(&c->rec_done[k], cudaEventDisableTiming) == cudaSuccess &&
                      cudaEventCreateWithFlags(&c->adj_done[k], cudaEventDisableTiming) == cudaSuccess;
             ok = ok && dev_alloc(&c->lam[0], lbytes) == cudaSuccess && dev_alloc(&c->lam[1], lbytes) == cudaSuccess &&
-                 dev_alloc(&c->aux, (size_t)lay.naux * lay.dstride * sizeof(T)) == cudaSuccess &&
-                 dev_alloc((void **)&c->slots, sizeof(double) * (adjoint_slots<T>(c->p.nx, c->p.ny) + 1)) == cudaSuccess;
+                 dev_alloc(&c->aux, (size_t)naux * lay.dstride * sizeof(T)) == cudaSuccess &&
+                 dev_alloc((void **)&c->slots, sizeof(double) * (tape_slots<T>(c) + 1)) == cudaSuccess;
+            if (ok && tape_wide(c) && !is_cdm(c))
+                ok = dev_alloc(&c->asums, wide_sums_bytes(c->p.nx, c->p.ny)) == cudaSuccess;
             if (!ok) {
                 free_tape(c);
                 return fail(c, LBM_E_NOMEM, "not enough device memory for the reverse sweep buffers");
@@ -591,20 +612,20 @@ lbm_status tape_forward(lbm_ctx *c, const T *rho0, int nsteps, int C, T *rhoT) {
     // What the reverse sweep needs of the last two segments goes straight
     // into their slots, so the sweep starts with no recompute: segment k's
     // stencil fields of states k C .. in slot k % kTapeSlots, and its states
-    // k C + 1 .. (single-pass contexts: the records of states k C .., the
+    // k C + 1 .. (contexts with a record: the records of states k C .., the
     // states themselves staying in the scratch pair).
     const int K = (nsteps - 1) / C, t0 = K * C, sl = K % kTapeSlots, nseg = C > 1 ? C - 1 : 0;
     const int slp = (K + kTapeSlots - 1) % kTapeSlots;   // the slot of segment K - 1
     const int tp = K >= 1 ? t0 - C : t0;   // the first step of the taped segments
     auto fbuf = [&](int t) -> void * {   // where state t (>= 1) goes
         if (t % C == 0) return c->ckpt[t / C];
-        if (!tape_fused(c) && t > t0 && t < nsteps) return c->seg[sl * nseg + (t - t0 - 1)];
-        if (!tape_fused(c) && t > tp && t < t0) return c->seg[slp * nseg + (t - tp - 1)];
+        if (!tape_rec(c) && t > t0 && t < nsteps) return c->seg[sl * nseg + (t - t0 - 1)];
+        if (!tape_rec(c) && t > tp && t < t0) return c->seg[slp * nseg + (t - tp - 1)];
         return c->tmp[t & 1];
     };
-    auto rbuf = [&](int t) -> float * {   // where the record of state t goes (single-pass)
-        if (!tape_fused(c) || t < tp) return nullptr;
-        return (float *)c->seg[((t / C) % kTapeSlots) * C + t % C];
+    auto rbuf = [&](int t) -> void * {   // where the record of state t goes
+        if (!tape_rec(c) || t < tp) return nullptr;
+        return c->seg[((t / C) % kTapeSlots) * C + t % C];
     };
     auto qbuf = [&](int t) -> void * {   // the stencil field of state t
         if (t >= t0 && t < nsteps) return c->segq[sl * C + (t - t0)];
@@ -653,19 +674,19 @@ lbm_status tape_backward(lbm_ctx *c, const T *grad_rhoT, T *grad_rho0, double *g
     // stencil fields: the single-pass layout (padded rows) or the plain one
     const int qpitch = tape_fused(c) ? fused_q_pitch(nx) : nx;
     const int qoff = (qpitch - nx) / 2;
-    const int nslots = adjoint_slots<T>(nx, ny);
+    const int nslots = tape_slots<T>(c);
     void **lam = c->lam, *aux = c->aux;
     double *slots = c->slots;
     const int rows = tape_fused(c) ? seg_rows_of(c) : 0;
     const int nseg = C > 1 ? C - 1 : 0;
-    // slot sl: states (single-pass: records) seg[sl * nseg + j] (seg[sl * C + j]),
+    // slot sl: states seg[sl * nseg + j], or records seg[sl * C + j], and
     // stencil fields segq[sl * C + j]
     auto segf = [&](int sl, int j) { return c->seg[sl * nseg + j]; };
     auto segrec = [&](int sl, int j) { return c->seg[sl * C + j]; };
     auto segqf = [&](int sl, int j) { return c->segq[sl * C + j]; };
     // Recompute segment k from its checkpoint with the forward kernels on
     // stream s into slot sl: the stencil field of every state t0 .. t1-1, and
-    // the states t0+1 .. t1-1 (single-pass: the records of states t0 .. t1-1,
+    // the states t0+1 .. t1-1 (with a record: the records of states t0 .. t1-1,
     // which takes the segment's last step too; the states pass through the
     // scratch pair).
     auto recompute = [&](int k, int sl, cudaStream_t s) {
@@ -692,8 +713,13 @@ lbm_status tape_backward(lbm_ctx *c, const T *grad_rhoT, T *grad_rho0, double *g
         const void *cur = c->ckpt[k];
         for (int t = t0; t < t1 && r == cudaSuccess; ++t) {
             r = tape_potential<T>(c, m, cur, segqf(sl, t - t0), s);
-            if (r == cudaSuccess && t < t1 - 1) {
-                r = tape_collide<T>(c, m, cur, segqf(sl, t - t0), segf(sl, t - t0), s);
+            if (r != cudaSuccess) break;
+            if (tape_wide(c)) {   // (the segment's last step too: its record)
+                void *dst = c->tmp[(t + 1) & 1];
+                r = tape_collide<T>(c, m, cur, segqf(sl, t - t0), dst, segrec(sl, t - t0), s);
+                cur = dst;
+            } else if (t < t1 - 1) {
+                r = tape_collide<T>(c, m, cur, segqf(sl, t - t0), segf(sl, t - t0), nullptr, s);
                 cur = segf(sl, t - t0);
             }
         }
@@ -731,7 +757,16 @@ lbm_status tape_backward(lbm_ctx *c, const T *grad_rhoT, T *grad_rho0, double *g
         if (e == cudaSuccess) e = cudaStreamWaitEvent(as, c->rec_done[sl], 0);
         const int t0 = k * C, t1 = std::min(N, t0 + C);
         for (int t = t1 - 1; t >= t0 && e == cudaSuccess; --t) {
-            const T *ft = (const T *)(tape_fused(c) ? segrec(sl, t - t0) : (t == t0 ? c->ckpt[k] : segf(sl, t - t0 - 1)));
+            const T *ft = (const T *)(tape_rec(c) ? segrec(sl, t - t0) : (t == t0 ? c->ckpt[k] : segf(sl, t - t0 - 1)));
+            if constexpr (std::is_same_v<T, double>) {
+                if (tape_wide(c)) {
+                    e = launch_wide_adjoint(m, R, aalp, is_sc(c), is_cdm(c), ft, (const double *)segqf(sl, t - t0),
+                                            (const double *)lam[li], (double *)aux, c->asums, (double *)lam[1 - li], slots,
+                                            /*overlap_prev=*/t != t1 - 1, as);
+                    li = 1 - li;
+                    continue;
+                }
+            }
             e = launch_adjoint_step<T>(m, R, aalp, is_sc(c), is_cdm(c), tau1, tape_fused(c), lay, ft,
                                        (const T *)segqf(sl, t - t0), qpitch, qoff, (const T *)lam[li], (T *)aux,
                                        (T *)lam[1 - li], slots, c->err, /*overlap_prev=*/t != t1 - 1, as);

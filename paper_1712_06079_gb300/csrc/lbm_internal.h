@@ -102,6 +102,18 @@ template <typename TS>
 cudaError_t launch_wide_moments(const Model<double> &m, bool sc, bool cdm, const TS *f, const double *q, double *sums,
                                 TS *rho, TS *vx, TS *vy, cudaStream_t s);
 
+// The reverse mode of FP64 lattices on that step (periodic): pass 2 with the
+// record of f (five planes of nx ny: rho, jx, jy, Dx, Dy), and one reverse step
+// from lambda(t+1) and the record and field of state t.  lambda has three planes
+// (rho_bar, j_bar) for tau = 1, else nine; aux five, else seven; sums holds the
+// block sums of D_bar (wide_sums_bytes); Tpart wide_adjoint_slots FP64 slots.
+cudaError_t launch_wide_collide_rec(const Model<double> &m, bool sc, bool cdm, const double *f, const double *q,
+                                    double *sums, double *fout, double *rec, cudaStream_t s);
+int wide_adjoint_slots(int nx, int ny);
+cudaError_t launch_wide_adjoint(const Model<double> &m, double R, double aalp, bool sc, bool cdm, const double *rec,
+                                const double *q, const double *lam, double *aux, double *sums, double *lam_out,
+                                double *Tpart, bool overlap_prev, cudaStream_t s);
+
 // HDM (Eq. 20) or CDM (Eq. 15 times 1/c_s^2) gradient of the periodic field
 // q (nx * ny, row-major) on a grid of spacing h into gx, gy.
 template <typename T>

@@ -118,6 +118,98 @@ __device__ __forceinline__ double carry_into(const double *own, const double *ot
     return acc;
 }
 
+// Block sums of a tile's fields: of `col` along its columns (warp 0), of `row`
+// along its rows (warp 1); lanes 0 .. 15 form BS, 16 .. 31 BT.
+__device__ __forceinline__ void write_block_sums(const WideArgs &A, const double (&col_f)[TY][TX + 1],
+                                                 const double (&row_f)[TY][TX + 1], int tx, int ty) {
+    const int nx = A.m.nx, ny = A.m.ny, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool fwd = lane < 16;
+    if (warp == 0) {
+        const int col = lane & 15, xc = tx * TX + col;
+        const int h = min(TY, ny - ty * TY);
+        if (xc < nx) {
+            double a = 0.0;
+            if (h == TY) {
+#pragma unroll
+                for (int k = 0; k < TY; ++k) a = fma(A.r, a, col_f[fwd ? k : TY - 1 - k][col]);
+            } else {
+                for (int k = 0; k < h; ++k) a = fma(A.r, a, col_f[fwd ? k : h - 1 - k][col]);
+            }
+            const long long o = (long long)ty * nx + xc;
+            if (in_bounds(o, A.nys, A.m.chk)) (fwd ? A.ys : A.yt)[o] = a;
+        }
+    } else if (warp == 1) {       // 8 rows x 2 blocks
+        const int row = lane & 7, b = (lane >> 3) & 1, yc = ty * TY + row, bx = 2 * tx + b;
+        const int w = min(BK, nx - bx * BK);
+        if (yc < ny && w > 0) {
+            const double *s = row_f[row] + b * BK;
+            double a = 0.0;
+            if (w == BK) {
+#pragma unroll
+                for (int k = 0; k < BK; ++k) a = fma(A.r, a, s[fwd ? k : BK - 1 - k]);
+            } else {
+                for (int k = 0; k < w; ++k) a = fma(A.r, a, s[fwd ? k : w - 1 - k]);
+            }
+            const long long o = (long long)yc * A.nbx + bx;
+            if (in_bounds(o, A.nxs, A.m.chk)) (fwd ? A.xs : A.xt)[o] = a;
+        }
+    }
+}
+
+// The sum that enters this thread's block (warp 0: a column's, lanes 0 .. 15 S
+// from below, 16 .. 31 T from above; warp 1: a row's, 8 rows x 2 blocks); 0 elsewhere.
+template <bool WALLS>
+__device__ __forceinline__ double tile_carry(const WideArgs &A, int tx, int ty) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool fwd = lane < 16;
+    if (warp == 0) {
+        const int xc = tx * TX + (lane & 15);
+        if (xc < A.m.nx)
+            return carry_into<WALLS>((fwd ? A.ys : A.yt) + xc, (fwd ? A.yt : A.ys) + xc, A.m.nx, ty, fwd ? -1 : 1, A.nby,
+                                     A.kby, A.r8, A.ryl, A.nys - xc, A.m.chk);
+    } else if (warp == 1) {
+        const int yc = ty * TY + (lane & 7), bx = 2 * tx + ((lane >> 3) & 1);
+        if (yc < A.m.ny && bx < A.nbx) {
+            const long long o = (long long)yc * A.nbx;
+            return carry_into<false>((fwd ? A.xs : A.xt) + o, (fwd ? A.xt : A.xs) + o, 1, bx, fwd ? -1 : 1, A.nbx,
+                                     A.kbx, A.r8, A.rxl, A.nxs - o, A.m.chk);
+        }
+    }
+    return 0.0;
+}
+
+// S_(i-1) and T_(i+1) of a tile's cells.
+struct TileSums {
+    double YS[TY][TX], YT[TY][TX];           // along the columns
+    double XS[TY][TX + 1], XT[TY][TX + 1];   // along the rows
+};
+
+// Steps S (lanes 0 .. 15) and T (16 .. 31) through the tile's blocks, warp 0 the
+// columns of colf, warp 1 the rows of rowf (staged with one cell around the
+// tile), from the entering sums; one code path for both directions.
+template <bool ABS>
+__device__ __forceinline__ void tile_step(const WideArgs &A, int tx, int ty, double carry,
+                                          const double (&colf)[TY + 2][TX + 2], const double (&rowf)[TY + 2][TX + 2],
+                                          TileSums &M) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp >= 2) return;
+    const bool fwd = lane < 16;
+    const int line = warp == 0 ? lane & 15 : lane & 7, b = warp == 0 ? 0 : (lane >> 3) & 1;
+    const int len = min(BK, warp == 0 ? A.m.ny - ty * TY : A.m.nx - (2 * tx + b) * BK);   // cells of the block
+    const double *src = warp == 0 ? &colf[1][line + 1] : &rowf[line + 1][b * BK + 1];
+    double *dst = warp == 0 ? &(fwd ? M.YS : M.YT)[0][line] : &(fwd ? M.XS : M.XT)[line][b * BK];
+    const int step = warp == 0 ? TX + 2 : 1, dstep = warp == 0 ? TX : 1;
+    double v = carry;
+#pragma unroll
+    for (int k = 0; k < BK; ++k) {
+        const int i = fwd ? k : len - 1 - k;
+        if (k < len) {
+            dst[i * dstep] = v;
+            if (k + 1 < BK) v = fma(A.r, v, ABS ? fabs(src[i * step]) : src[i * step]);
+        }
+    }
+}
+
 // Pass 1: rho (Eq. 3), the potential field q (Eq. 8 / 21) and, for the HDM, the
 // block sums of the stencil's field (Phi = |q| for Shan-Chen, U for Zhang-Chen).
 template <typename TS, bool HDM>
@@ -152,50 +244,19 @@ __global__ void __launch_bounds__(NT) wide_potential_kernel(const __grid_constan
     if (!HDM) return;
     S[ly][lx] = phi;
     __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool fwd = lane < 16;   // BS, else BT
-    if (warp == 0) {              // columns
-        const int col = lane & 15, xc = tx * TX + col;
-        const int h = min(TY, ny - ty * TY);
-        if (xc < nx) {
-            double a = 0.0;
-            if (h == TY) {
-#pragma unroll
-                for (int k = 0; k < TY; ++k) a = fma(A.r, a, S[fwd ? k : TY - 1 - k][col]);
-            } else {
-                for (int k = 0; k < h; ++k) a = fma(A.r, a, S[fwd ? k : h - 1 - k][col]);
-            }
-            const long long o = (long long)ty * nx + xc;
-            if (in_bounds(o, A.nys, m.chk)) (fwd ? A.ys : A.yt)[o] = a;
-        }
-    } else if (warp == 1) {       // rows: 8 rows x 2 blocks
-        const int row = lane & 7, b = (lane >> 3) & 1, yc = ty * TY + row, bx = 2 * tx + b;
-        const int w = min(BK, nx - bx * BK);
-        if (yc < ny && w > 0) {
-            const double *s = S[row] + b * BK;
-            double a = 0.0;
-            if (w == BK) {
-#pragma unroll
-                for (int k = 0; k < BK; ++k) a = fma(A.r, a, s[fwd ? k : BK - 1 - k]);
-            } else {
-                for (int k = 0; k < w; ++k) a = fma(A.r, a, s[fwd ? k : w - 1 - k]);
-            }
-            const long long o = (long long)yc * A.nbx + bx;
-            if (in_bounds(o, A.nxs, m.chk)) (fwd ? A.xs : A.xt)[o] = a;
-        }
-    }
+    write_block_sums(A, S, S, tx, ty);
 }
 
 // Pass 2: gradient of q, force (Eq. 22 / 7), exact-difference forcing with BGK
-// (Eq. 1, 2, 10) and push streaming; MOM: rho and the Eq. 11 velocity instead.
-template <typename TS, bool SC, bool HDM, bool TAU1, bool WALLS, bool MOM>
+// (Eq. 1, 2, 10) and push streaming; MOM: rho and the Eq. 11 velocity instead;
+// REC: also the reverse mode's record of f, planes rho, jx, jy, Dx, Dy at rho_out.
+template <typename TS, bool SC, bool HDM, bool TAU1, bool WALLS, bool MOM, bool REC = false>
 __global__ void __launch_bounds__(NT) wide_collide_kernel(const __grid_constant__ WideArgs A, const TS *f,
                                                           const double *q, TS *fout, TS *rho_out, TS *vx_out,
                                                           TS *vy_out) {
     constexpr int QW = TX + 2, QH = TY + 2;
     __shared__ double Q[QH][QW];                          // q over the tile and one cell around it
-    __shared__ double YS[TY][TX], YT[TY][TX];             // S_(y-1), T_(y+1) along the column
-    __shared__ double XS[TY][TX + 1], XT[TY][TX + 1];     // S_(x-1), T_(x+1) along the row
+    __shared__ TileSums M;
     const Model<double> &m = A.m;
     const int nx = m.nx, ny = m.ny;
     const long long n = (long long)nx * ny;
@@ -205,7 +266,6 @@ __global__ void __launch_bounds__(NT) wide_collide_kernel(const __grid_constant_
     const int x = x0 + lx, y = y0 + ly;
     const bool valid = x < nx && y < ny;
     const long long c = (long long)min(y, ny - 1) * nx + min(x, nx - 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     ptx::griddep_wait();   // pass 1 has written q and the block sums
 
     // the rows and columns of the tile's halo: periodic, or mirrored across a wall
@@ -217,43 +277,13 @@ __global__ void __launch_bounds__(NT) wide_collide_kernel(const __grid_constant_
         const long long g = (long long)py * nx + px;
         Q[ry][rx] = in_bounds(g, n, m.chk) ? q[g] : 0.0;
     }
-    // warps 0 and 1: the sums that enter the tile's blocks (columns; rows)
-    const bool fwd = lane < 16;
-    double carry = 0.0;
-    if (HDM && warp == 0) {
-        const int xc = x0 + (lane & 15);
-        if (xc < nx)
-            carry = carry_into<WALLS>((fwd ? A.ys : A.yt) + xc, (fwd ? A.yt : A.ys) + xc, nx, ty, fwd ? -1 : 1, A.nby,
-                                      A.kby, A.r8, A.ryl, A.nys - xc, m.chk);
-    } else if (HDM && warp == 1) {
-        const int yc = y0 + (lane & 7), bx = 2 * tx + ((lane >> 3) & 1);
-        if (yc < ny && bx < A.nbx) {
-            const long long o = (long long)yc * A.nbx;
-            carry = carry_into<false>((fwd ? A.xs : A.xt) + o, (fwd ? A.xt : A.xs) + o, 1, bx, fwd ? -1 : 1, A.nbx,
-                                      A.kbx, A.r8, A.rxl, A.nxs - o, m.chk);
-        }
-    }
+    const double carry = HDM ? tile_carry<WALLS>(A, tx, ty) : 0.0;
     double fi[kQ];
 #pragma unroll
     for (int i = 0; i < kQ; ++i) fi[i] = in_bounds(i * n + c, kQ * n, m.chk) ? (double)f[i * n + c] : 0.0;
     __syncthreads();
     auto mag = [](double v) { return SC ? fabs(v) : v; };
-    if (HDM && warp < 2) {   // S upwards (lanes 0 .. 15), T downwards, one code path for both
-        const int line = warp == 0 ? lane & 15 : lane & 7, b = warp == 0 ? 0 : (lane >> 3) & 1;
-        const int len = min(BK, warp == 0 ? ny - y0 : nx - (2 * tx + b) * BK);   // cells of the block
-        const double *src = warp == 0 ? &Q[1][line + 1] : &Q[line + 1][b * BK + 1];
-        double *dst = warp == 0 ? &(fwd ? YS : YT)[0][line] : &(fwd ? XS : XT)[line][b * BK];
-        const int step = warp == 0 ? QW : 1, dstep = warp == 0 ? TX : 1;
-        double v = carry;
-#pragma unroll
-        for (int k = 0; k < BK; ++k) {
-            const int i = fwd ? k : len - 1 - k;
-            if (k < len) {
-                dst[i * dstep] = v;
-                if (k + 1 < BK) v = fma(A.r, v, mag(src[i * step]));
-            }
-        }
-    }
+    if (HDM) tile_step<SC>(A, tx, ty, carry, Q, Q, M);
     // moments (Eq. 3) from the sums over the populations moving east, west, north, south
     const double east = fi[1] + fi[5] + fi[8], west = fi[3] + fi[6] + fi[7];
     const double r = fi[0] + fi[2] + fi[4] + east + west;
@@ -266,8 +296,8 @@ __global__ void __launch_bounds__(NT) wide_collide_kernel(const __grid_constant_
     const double *p = &Q[ly + 1][lx + 1];
     double dx, dy;
     if (HDM) {
-        dx = fma(A.c1, mag(p[1]) - mag(p[-1]), A.cs * (XT[ly][lx] - XS[ly][lx]));
-        dy = fma(A.c1, mag(p[QW]) - mag(p[-QW]), A.cs * (YT[ly][lx] - YS[ly][lx]));
+        dx = fma(A.c1, mag(p[1]) - mag(p[-1]), A.cs * (M.XT[ly][lx] - M.XS[ly][lx]));
+        dy = fma(A.c1, mag(p[QW]) - mag(p[-QW]), A.cs * (M.YT[ly][lx] - M.YS[ly][lx]));
     } else {   // Eq. 15 times 1/c_s^2
         const double ne = mag(p[QW + 1]), nw = mag(p[QW - 1]), se = mag(p[-QW + 1]), sw = mag(p[-QW - 1]);
         dx = (1.0 / 3.0) * (mag(p[1]) - mag(p[-1])) + (1.0 / 12.0) * ((ne + se) - (nw + sw));
@@ -281,6 +311,12 @@ __global__ void __launch_bounds__(NT) wide_collide_kernel(const __grid_constant_
     } else {    // Eq. 7
         Fx = -dx;
         Fy = -dy;
+    }
+    if constexpr (REC) {
+        const double v[5] = {r, jx, jy, dx, dy};
+#pragma unroll
+        for (int k = 0; k < 5; ++k)
+            if (in_bounds(k * n + c, 5 * n, m.chk)) rho_out[k * n + c] = v[k];
     }
     if (MOM) {  // Eq. 3 and Eq. 11
         if (in_bounds(c, n, m.chk)) {
@@ -333,6 +369,268 @@ __global__ void __launch_bounds__(NT) wide_collide_kernel(const __grid_constant_
     if (in_bounds(c, kQ * n, m.chk)) fout[c] = (TS)(r - moved);
 }
 
+// ---- reverse step (the adjoint of the step, as adjoint.cu derives it) ----
+//
+// From the record of the state (rho, j, and the derivatives D the forward used)
+// and its field q, kernel A does the local adjoint of the forcing and collision
+// and writes D_bar with its block sums, the partial rho_bar, and kappa, theta =
+// dPhi/dU (dU/drho, dU/dtheta); kernel B differentiates D_bar (the transposed
+// derivative is its negative) and finishes rho_bar, T_bar and lambda(t).  Both are
+// bound by FP64 instructions as the forward passes are, so the directions are
+// taken in opposite pairs (sums and differences of g), Phi comes from the stored
+// field instead of a square root, and kappa and theta are formed once.  16 steps
+// forward and back at 256^2: 2.70 ms with the kernels that differentiate the field
+// and D_bar by the direct radius-40 stencil on 32 x 16 tiles, 1.64 ms with these.
+struct WideAdjArgs {
+    WideArgs w;                // (its block sums: those of D_bar)
+    double R, aalp;            // gas constant, a dalpha/dT
+    const double *rec, *q;     // record of the state (five planes) and its field
+    const double *lam;         // lambda(t+1): three planes for tau = 1, else nine
+    double *lam_out;           // lambda(t)
+    double *aux;               // D_bar_x, D_bar_y, rho_bar, kappa, theta[, j_bar_x, j_bar_y]
+    double *Tpart;             // one FP64 slot per warp of A, then of B
+};
+
+// dU/drho and dU/dtheta (theta = T, or G for the effective mass of Eq. 4-5) times
+// dPhi/dU = s / (2 Phi) (Shan-Chen, q = s Phi) or 1; U of Eq. 8 with Eq. 24, 27-29.
+template <bool SC>
+__device__ __forceinline__ void wide_eos(const WideAdjArgs &a, double rho, double q, double &kappa, double &theta) {
+    const Model<double> &m = a.w.m;
+    double dr, dt;
+    if (m.eos == LBM_EOS_PSI_EXP) {
+        const double e = exp(-rho * m.b), psi = 1.0 - e;
+        dr = 2.0 * m.a * psi * e * m.b;
+        dt = 0.5 * psi * psi;
+    } else {
+        double dpdr, dpdT;
+        if (m.eos == LBM_EOS_CS) {
+            const double e = m.b * rho * 0.25, om = 1.0 - e, inv = 1.0 / om, inv3 = inv * inv * inv;
+            const double num = fma(e, fma(e, om, 1.0), 1.0);   // 1 + e + e^2 - e^3
+            const double Z = num * inv3, dZ = fma(fma(e, fma(-3.0, e, 2.0), 1.0), om, 3.0 * num) * inv3 * inv;
+            dpdr = fma(m.RT, fma(e, dZ, Z), -2.0 * m.a * rho);
+            dpdT = a.R * rho * Z;
+        } else {
+            const double inv = 1.0 / (1.0 - m.b * rho), ri = rho * inv;
+            dpdr = m.RT * inv * inv;
+            dpdT = a.R * ri;
+            if (m.eos == LBM_EOS_VDW) {
+                dpdr = fma(-2.0 * m.a, rho, dpdr);
+            } else if (m.eos == LBM_EOS_PR) {
+                const double br = m.b * rho, id = 1.0 / fma(br, 2.0 - br, 1.0), rid = rho * id;
+                dpdr -= 2.0 * m.aal * (1.0 + br) * rid * id;
+                dpdT -= a.aalp * rho * rid;
+            } else {   // RK, RKS
+                const double br = m.b * rho, id = 1.0 / (1.0 + br), rid = rho * id;
+                dpdr -= m.aal * (2.0 + br) * rid * id;
+                dpdT -= a.aalp * rho * rid;
+            }
+        }
+        dr = fma(m.k, dpdr, -1.0 / 3.0);
+        dt = m.k * dpdT;
+    }
+    const double d = SC ? (q != 0.0 ? 0.5 / q : 0.0) : 1.0;   // s / (2 Phi) = 1 / (2 q)
+    kappa = d * dr;
+    theta = d * dt;
+}
+
+// Sum over the warp, added to the warp's own slot (one writer per slot and
+// launch, the launches ordered: reproducible).
+__device__ __forceinline__ void wide_slot_add(double v, double *part) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(part + (size_t)blockIdx.x * (NT / 32) + (threadIdx.x >> 5), v);
+}
+
+template <bool SC, bool HDM, bool TAU1>
+__global__ void __launch_bounds__(NT) wide_adj_a_kernel(const __grid_constant__ WideAdjArgs a) {
+    __shared__ double L[TAU1 ? 3 : 1][TY + 2][TX + 2];   // lambda with one cell around the tile
+    __shared__ double SX[TY][TX + 1], SY[TY][TX + 1];    // D_bar
+    const WideArgs &A = a.w;
+    const Model<double> &m = A.m;
+    const int nx = m.nx, ny = m.ny;
+    const long long n = (long long)nx * ny;
+    const int ty = blockIdx.x / A.ntx, tx = blockIdx.x - ty * A.ntx;
+    const int lx = threadIdx.x & (TX - 1), ly = threadIdx.x / TX, x = tx * TX + lx, y = ty * TY + ly;
+    const bool valid = x < nx && y < ny;
+    const int xc = min(x, nx - 1), yc = min(y, ny - 1);
+    const long long c = (long long)yc * nx + xc;
+    ptx::griddep_wait();
+    auto rec = [&](int k) { return in_bounds(k * n + c, 5 * n, m.chk) ? a.rec[k * n + c] : 1.0; };
+    const double r = rec(0), jx = rec(1), jy = rec(2), Dx = rec(3), Dy = rec(4);
+    const double q = in_bounds(c, n, m.chk) ? a.q[c] : 1.0;
+    double g[kQ];   // g_i = lambda_i(x + e_i)
+    if (TAU1) {
+        for (int k = threadIdx.x; k < 3 * (TY + 2) * (TX + 2); k += NT) {
+            const int f = k / ((TY + 2) * (TX + 2)), kk = k - f * ((TY + 2) * (TX + 2));
+            const int ry = kk / (TX + 2), rx = kk - ry * (TX + 2);
+            const int gx = min(tx * TX - 1 + rx, nx), gy = min(ty * TY - 1 + ry, ny);
+            const long long o = f * n + (long long)(gy < 0 ? ny - 1 : (gy == ny ? 0 : gy)) * nx +
+                                (gx < 0 ? nx - 1 : (gx == nx ? 0 : gx));
+            L[f][ry][rx] = in_bounds(o, 3 * n, m.chk) ? a.lam[o] : 0.0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kQ; ++i) {   // lambda_i = rho_bar + e_i . j_bar
+            double v = L[0][ly + 1 + ey(i)][lx + 1 + ex(i)];
+            if (ex(i) == 1) v += L[TAU1 ? 1 : 0][ly + 1 + ey(i)][lx + 1 + ex(i)];
+            if (ex(i) == -1) v -= L[TAU1 ? 1 : 0][ly + 1 + ey(i)][lx + 1 + ex(i)];
+            if (ey(i) == 1) v += L[TAU1 ? 2 : 0][ly + 1 + ey(i)][lx + 1 + ex(i)];
+            if (ey(i) == -1) v -= L[TAU1 ? 2 : 0][ly + 1 + ey(i)][lx + 1 + ex(i)];
+            g[i] = v;
+        }
+    } else {
+        const int xp = xc + 1 == nx ? 0 : xc + 1, xm = xc == 0 ? nx - 1 : xc - 1;
+        const int yp = yc + 1 == ny ? 0 : yc + 1, ym = yc == 0 ? ny - 1 : yc - 1;
+#pragma unroll
+        for (int i = 0; i < kQ; ++i) {
+            const long long o = i * n + (long long)(ey(i) == 1 ? yp : (ey(i) == -1 ? ym : yc)) * nx +
+                                (ex(i) == 1 ? xp : (ex(i) == -1 ? xm : xc));
+            g[i] = in_bounds(o, kQ * n, m.chk) ? a.lam[o] : 0.0;
+        }
+    }
+    double kappa, theta;
+    wide_eos<SC>(a, r, q, kappa, theta);
+    const double inv = 1.0 / r, ux = jx * inv, uy = jy * inv;
+    const double s = SC ? -2.0 * q : -1.0, Fx = s * Dx, Fy = s * Dy;   // Eq. 22 / 7
+    const double vx = fma(Fx, inv, ux), vy = fma(Fy, inv, uy);
+    // With f^eq_i(v) = w_i rho (a + e.v (3 + 4.5 e.v)), a = 1 - 1.5 |v|^2, the sums over
+    // the directions of g_i w_i times 1, e_i (3 + 9 e.v), e.v (3 + 4.5 e.v), a direction
+    // and its opposite at a time: gs, gd the sum and difference of their g.
+    double G0 = (4.0 / 9.0) * g[0], Gx = 0.0, Gy = 0.0, Rv = 0.0, Hx = 0.0, Hy = 0.0, Ru = 0.0;
+#pragma unroll
+    for (int cl = 0; cl < 2; ++cl) {   // the axes (w = 1/9), the diagonals (1/36)
+        double sg = 0.0, ax = 0.0, ay = 0.0, b = 0.0, hx = 0.0, hy = 0.0, bu = 0.0;
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+            const int i = cl == 0 ? 1 + d : 5 + d, o = opp(i);
+            const double gs = g[i] + g[o], g3 = 3.0 * (g[i] - g[o]);
+            auto along = [&](double px, double py) { return i == 1 ? px : (i == 2 ? py : (i == 5 ? px + py : py - px)); };
+            auto add = [&](double ev, double &sx, double &sy, double &sb) {
+                const double t = ev * gs, A1 = fma(9.0, t, g3);
+                if (ex(i) == 1) sx += A1;
+                if (ex(i) == -1) sx -= A1;
+                if (ey(i) == 1) sy += A1;
+                sb = fma(ev, fma(4.5, t, g3), sb);
+            };
+            sg += gs;
+            add(along(vx, vy), ax, ay, b);
+            if (!TAU1) add(along(ux, uy), hx, hy, bu);
+        }
+        const double w = cl == 0 ? 1.0 / 9.0 : 1.0 / 36.0;
+        G0 = fma(w, sg, G0);
+        Gx = fma(w, ax, Gx);
+        Gy = fma(w, ay, Gy);
+        Rv = fma(w, b, Rv);
+        if (!TAU1) {
+            Hx = fma(w, hx, Hx);
+            Hy = fma(w, hy, Hy);
+            Ru = fma(w, bu, Ru);
+        }
+    }
+    double rb = fma(fma(-1.5, fma(vx, vx, vy * vy), 1.0), G0, Rv);
+    const double vbx = r * fma(-3.0 * vx, G0, Gx), vby = r * fma(-3.0 * vy, G0, Gy);
+    double ubx = vbx, uby = vby;
+    if (!TAU1) {   // the f^eq(u) terms enter with the weights -(1 - omega) g_i
+        const double om1 = 1.0 - m.omega;
+        rb -= om1 * fma(fma(-1.5, fma(ux, ux, uy * uy), 1.0), G0, Ru);
+        ubx -= om1 * r * fma(-3.0 * ux, G0, Hx);
+        uby -= om1 * r * fma(-3.0 * uy, G0, Hy);
+    }
+    const double Fbx = vbx * inv, Fby = vby * inv, jbx = ubx * inv, jby = uby * inv;
+    rb -= fma(Fbx, Fx, Fby * Fy) * inv;
+    rb -= fma(jbx, ux, jby * uy);
+    const double Dbx = s * Fbx, Dby = s * Fby;
+    double tacc = 0.0;
+    if (SC) {   // the centre factor Phi of F = -2 s Phi D
+        const double pc = (q >= 0.0 ? -2.0 : 2.0) * fma(Fbx, Dx, Fby * Dy);
+        rb = fma(pc, kappa, rb);
+        tacc = valid ? pc * theta : 0.0;
+    }
+    if (HDM) {
+        SX[ly][lx] = valid ? Dbx : 0.0;
+        SY[ly][lx] = valid ? Dby : 0.0;
+        __syncthreads();
+    }
+    ptx::griddep_launch_dependents();
+    if (valid) {
+        const double v[7] = {Dbx, Dby, rb, kappa, theta, jbx, jby};
+#pragma unroll
+        for (int k = 0; k < (TAU1 ? 5 : 7); ++k)
+            if (in_bounds(k * n + c, 7 * n, m.chk)) a.aux[k * n + c] = v[k];
+        if (TAU1 && in_bounds(2 * n + c, 3 * n, m.chk)) {
+            a.lam_out[n + c] = jbx;
+            a.lam_out[2 * n + c] = jby;
+        }
+    }
+    if (HDM) write_block_sums(A, SY, SX, tx, ty);
+    if (SC) wide_slot_add(tacc, a.Tpart);
+}
+
+template <bool HDM, bool TAU1>
+__global__ void __launch_bounds__(NT) wide_adj_b_kernel(const __grid_constant__ WideAdjArgs a) {
+    __shared__ double QX[TY + 2][TX + 2], QY[TY + 2][TX + 2];   // D_bar with one cell around the tile
+    __shared__ TileSums M;
+    const WideArgs &A = a.w;
+    const Model<double> &m = A.m;
+    const int nx = m.nx, ny = m.ny;
+    const long long n = (long long)nx * ny;
+    const int ty = blockIdx.x / A.ntx, tx = blockIdx.x - ty * A.ntx;
+    const int lx = threadIdx.x & (TX - 1), ly = threadIdx.x / TX, x = tx * TX + lx, y = ty * TY + ly;
+    const bool valid = x < nx && y < ny;
+    const int xc = min(x, nx - 1), yc = min(y, ny - 1);
+    const long long c = (long long)yc * nx + xc;
+    ptx::griddep_wait();   // A's output
+    for (int k = threadIdx.x; k < (TY + 2) * (TX + 2); k += NT) {
+        const int ry = k / (TX + 2), rx = k - ry * (TX + 2);
+        const int gx = min(tx * TX - 1 + rx, nx), gy = min(ty * TY - 1 + ry, ny);
+        const long long o = (long long)(gy < 0 ? ny - 1 : (gy == ny ? 0 : gy)) * nx + (gx < 0 ? nx - 1 : (gx == nx ? 0 : gx));
+        QX[ry][rx] = in_bounds(o, n, m.chk) ? a.aux[o] : 0.0;
+        QY[ry][rx] = in_bounds(o, n, m.chk) ? a.aux[n + o] : 0.0;
+    }
+    const double carry = HDM ? tile_carry<false>(A, tx, ty) : 0.0;
+    auto aux = [&](int k) { return in_bounds(k * n + c, 7 * n, m.chk) ? a.aux[k * n + c] : 0.0; };
+    const double rb0 = aux(2), kappa = aux(3), theta = aux(4);
+    __syncthreads();
+    if (HDM) {
+        tile_step<false>(A, tx, ty, carry, QY, QX, M);
+        __syncthreads();
+    }
+    ptx::griddep_launch_dependents();
+    const double *px = &QX[ly + 1][lx + 1], *py = &QY[ly + 1][lx + 1];
+    constexpr int QW = TX + 2;
+    double dd;   // Dx[D_bar_x] + Dy[D_bar_y]
+    if (HDM) {
+        dd = fma(A.c1, (px[1] - px[-1]) + (py[QW] - py[-QW]),
+                 A.cs * ((M.XT[ly][lx] - M.XS[ly][lx]) + (M.YT[ly][lx] - M.YS[ly][lx])));
+    } else {
+        dd = (1.0 / 3.0) * ((px[1] - px[-1]) + (py[QW] - py[-QW])) +
+             (1.0 / 12.0) * (((px[QW + 1] + px[-QW + 1]) - (px[QW - 1] + px[-QW - 1])) +
+                             ((py[QW + 1] + py[QW - 1]) - (py[-QW + 1] + py[-QW - 1])));
+    }
+    const double rb = fma(-kappa, dd, rb0);
+    if (valid) {
+        if (TAU1) {
+            if (in_bounds(c, 3 * n, m.chk)) a.lam_out[c] = rb;
+        } else {
+            const double jbx = aux(5), jby = aux(6), om1 = 1.0 - m.omega;
+            const int xp = x + 1 == nx ? 0 : x + 1, xm = x == 0 ? nx - 1 : x - 1;
+            const int yp = y + 1 == ny ? 0 : y + 1, ym = y == 0 ? ny - 1 : y - 1;
+#pragma unroll
+            for (int i = 0; i < kQ; ++i) {
+                const long long o = i * n + (long long)(ey(i) == 1 ? yp : (ey(i) == -1 ? ym : y)) * nx +
+                                    (ex(i) == 1 ? xp : (ex(i) == -1 ? xm : x));
+                double li = fma(om1, in_bounds(o, kQ * n, m.chk) ? a.lam[o] : 0.0, rb);
+                if (ex(i) == 1) li += jbx;
+                if (ex(i) == -1) li -= jbx;
+                if (ey(i) == 1) li += jby;
+                if (ey(i) == -1) li -= jby;
+                if (in_bounds(i * n + c, kQ * n, m.chk)) a.lam_out[i * n + c] = li;
+            }
+        }
+    }
+    wide_slot_add(valid ? -theta * dd : 0.0, a.Tpart);
+}
+
 // Blocks that cover kReach cells of the cyclic (mirror: mirrored) line of n
 // cells, wherever the first of them lies.  Only starts near the short block at
 // the line's end need more than kReach / BK.
@@ -375,17 +673,21 @@ WideArgs args_of(const Model<double> &m, double *sums) {
 }
 
 template <typename K, typename... Args>
-cudaError_t launch_tiles(K kern, const WideArgs &a, cudaStream_t s, Args... args) {
+cudaError_t launch_grid(K kern, const WideArgs &w, bool pdl, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((long long)a.ntx * a.nby));
+    cfg.gridDim = dim3((unsigned)((long long)w.ntx * w.nby));
     cfg.blockDim = dim3(NT);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, a, args...);
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+template <typename K, typename... Args>
+cudaError_t launch_tiles(K kern, const WideArgs &w, cudaStream_t s, Args... args) {
+    return launch_grid(kern, w, true, s, w, args...);
 }
 
 template <typename TS, bool MOM>
@@ -438,6 +740,60 @@ template <typename TS>
 cudaError_t launch_wide_moments(const Model<double> &m, bool sc, bool cdm, const TS *f, const double *q, double *sums,
                                 TS *rho, TS *vx, TS *vy, cudaStream_t s) {
     return pick_collide<TS, true>(args_of(m, sums), sc, cdm, f, q, (TS *)nullptr, rho, vx, vy, s);
+}
+
+cudaError_t launch_wide_collide_rec(const Model<double> &m, bool sc, bool cdm, const double *f, const double *q,
+                                    double *sums, double *fout, double *rec, cudaStream_t s) {
+    const WideArgs a = args_of(m, sums);
+    const bool tau1 = m.omega == 1.0;
+    double *none = nullptr;
+#define LBM_REC(SC, HDM)                                                                                             \
+    return tau1 ? launch_tiles(wide_collide_kernel<double, SC, HDM, true, false, false, true>, a, s, f, q, fout, rec, none, none) \
+                : launch_tiles(wide_collide_kernel<double, SC, HDM, false, false, false, true>, a, s, f, q, fout, rec, none, none)
+    if (sc) {
+        if (cdm) LBM_REC(true, false);
+        LBM_REC(true, true);
+    }
+    if (cdm) LBM_REC(false, false);
+    LBM_REC(false, true);
+#undef LBM_REC
+}
+
+int wide_adjoint_slots(int nx, int ny) { return 2 * ((nx + TX - 1) / TX) * ((ny + TY - 1) / TY) * (NT / 32); }
+
+cudaError_t launch_wide_adjoint(const Model<double> &m, double R, double aalp, bool sc, bool cdm, const double *rec,
+                                const double *q, const double *lam, double *aux, double *sums, double *lam_out,
+                                double *Tpart, bool overlap_prev, cudaStream_t s) {
+    WideAdjArgs a{};
+    a.w = args_of(m, sums);
+    a.R = R;
+    a.aalp = aalp;
+    a.rec = rec;
+    a.q = q;
+    a.lam = lam;
+    a.lam_out = lam_out;
+    a.aux = aux;
+    a.Tpart = Tpart;
+    const bool tau1 = m.omega == 1.0;
+    void (*ka)(const WideAdjArgs), (*kb)(const WideAdjArgs);
+#define LBM_ADJ(HDM, TAU1)                                                                       \
+    do {                                                                                         \
+        ka = sc ? wide_adj_a_kernel<true, HDM, TAU1> : wide_adj_a_kernel<false, HDM, TAU1>;      \
+        kb = wide_adj_b_kernel<HDM, TAU1>;                                                       \
+    } while (0)
+    if (cdm) {
+        if (tau1) LBM_ADJ(false, true);
+        else LBM_ADJ(false, false);
+    } else {
+        if (tau1) LBM_ADJ(true, true);
+        else LBM_ADJ(true, false);
+    }
+#undef LBM_ADJ
+    // (A may overlap the previous step's B, but not an event wait on the recompute's stream)
+    cudaError_t e = launch_grid(ka, a.w, overlap_prev, s, a);
+    if (e != cudaSuccess) return e;
+    a.Tpart = Tpart + wide_adjoint_slots(m.nx, m.ny) / 2;
+    return launch_grid(kb, a.w, true, s, a);
 }
 
 #define LBM_WIDE_INST(TS)                                                                                          \

@@ -73,3 +73,35 @@ def test_a_requested_radius_keeps_its_truncation():
     scale = np.abs(out[0]).max()
     assert np.abs(out[40] - out[0]).max() < 1e-14 * scale * 100
     assert np.abs(out[8] - out[0]).max() > 1e-9 * scale
+
+
+@pytest.mark.parametrize("nx,ny", [(17, 9), (8, 33), (23, 41), (6, 100)])
+@pytest.mark.parametrize("eos,force,grad,tau", [("pr", "sc", "hdm", 1.0), ("rk", "zc", "hdm", 0.9), ("vdw", "sc", "cdm", 1.1),
+                                                ("cs", "zc", "cdm", 1.0)])
+def test_reverse_step_is_the_complex_step_derivative(nx, ny, eos, force, grad, tau):
+    # the FP64 reverse kernels on short and ragged lines, 5 steps with a
+    # checkpoint every 2 (a recomputed segment among them): 1e-11, the bar of the
+    # oracle's derivative on the larger lattices
+    torch = pytest.importorskip("torch")
+    t = inputs.EOS_TABLE[eos]
+    p = lbm.Params(nx=nx, ny=ny, eos=eos, a=t["a"], b=t["b"], omega=t["omega"], Tr=0.9, k=t["k"], tau=tau, force=force,
+                   grad=grad, prec="f64", stream=torch.cuda.current_stream().cuda_stream)
+    op = oracle.params_at(nx, ny, eos, t["a"], t["b"], 0.9, omega=t["omega"], k=t["k"], tau=tau, force=force, grad=grad)
+    g, l, _ = oracle.maxwell(op)
+    xi = inputs.uniform01(nx + 3 * ny, 3 * nx * ny).reshape(3, ny, nx)
+    rho0 = 0.5 * (g + l) * (1 + 0.1 * (xi[0] - 0.5))
+    v = xi[1] - 0.5                                # dL/drho_T
+    with lbm.Lattice(p) as lat:
+        x = torch.tensor(rho0, device="cuda")
+        rT, g0 = torch.empty_like(x), torch.empty_like(x)
+        gr = torch.tensor(v, device="cuda")
+        torch.cuda.synchronize()
+        lat.adjoint_forward(x.data_ptr(), 5, 2, rT.data_ptr())
+        _, gtr, _ = lat.adjoint_backward(gr.data_ptr(), g0.data_ptr())
+        out, grad0 = rT.cpu().numpy(), g0.cpu().numpy()
+    r, dT = oracle.tangent(op, rho0, 5, dTr=1.0)
+    assert np.max(np.abs(out / r - 1)) < 1e-12
+    assert abs(gtr - (v * dT).sum()) < 1e-11 * np.abs(v * dT).sum()
+    d = xi[2] - 0.5
+    _, dd = oracle.tangent(op, rho0, 5, drho0=d)
+    assert abs((grad0 * d).sum() - (v * dd).sum()) < 1e-11 * np.abs(v * dd).sum()
