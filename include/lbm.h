@@ -345,7 +345,10 @@ lbm_status lbm_batch_get_launch(lbm_batch *b, int *block_threads, int *grid_bloc
  * its narrowest slice at least as wide as its x halo (the HDM radius, 1 for
  * CDM), and both distribution buffers plus the haloed field of the widest
  * slice within a block's shared memory; otherwise LBM_E_INVALID and the batch
- * keeps its form.  cluster = 0 returns to the grid
+ * keeps its form.  (A batch of FP32 HDM
+ * lattices with rows of at least 53 cells needs less: one distribution buffer, and
+ * as many threads as a slice has groups of four cells, whatever block_threads is;
+ * the conditions are the same.)  cluster = 0 returns to the grid
  * form.  lbm_batch_get_launch then reports block_threads and cluster * n. */
 lbm_status lbm_batch_set_cluster(lbm_batch *b, int cluster, int block_threads);
 /* The batch's form: 0 grid, 2/4/8 the cluster form's cluster size, -1 grouped. */
@@ -370,7 +373,7 @@ lbm_status lbm_batch_get_cluster(lbm_batch *b, int *cluster);
 enum { LBM_GROUPS_BALANCED = -1 };
 lbm_status lbm_batch_set_groups(lbm_batch *b, int max_smem_bytes, int block_threads);
 /* Groups of the grouped form (ngroups = 0 otherwise): cluster size, instance
- * count and shared memory per CTA of each, largest cluster first; cluster,
+ * count and shared memory per CTA of each (as launched), largest cluster first; cluster,
  * count and smem_bytes may be NULL, else hold at least 3 entries. */
 lbm_status lbm_batch_get_groups(lbm_batch *b, int *ngroups, int *cluster, int *count, int *smem_bytes);
 

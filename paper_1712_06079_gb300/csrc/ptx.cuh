@@ -92,6 +92,12 @@ __device__ __forceinline__ void cp_async(void *smem_dst, const void *gmem_src) {
                  : "memory");
 }
 
+// The same for 16 bytes past L1 (cp.async.cg): data that other SMs write while
+// the kernel runs.
+__device__ __forceinline__ void cp_async16_l2(void *smem_dst, const void *gmem_src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem_dst)), "l"(gmem_src) : "memory");
+}
+
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Programmatic dependent launch (sm_90 and later).  launch_dependents lets the
