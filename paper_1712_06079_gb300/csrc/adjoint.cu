@@ -51,6 +51,7 @@
 // steps in the same slots, and over the slots in a fixed order at the end.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "lbm_internal.h"
@@ -59,14 +60,25 @@
 namespace lbm {
 namespace {
 
-template <typename T>
+// Tiles, two cells per thread.  On plain rows a tall tile: the direct stencil's y
+// halo is staged once per 16 rows.  In the padded FP32 layout 64 x 4, 128 threads:
+// 512^2 makes 1024 CTAs, about seven for every SM, where 16 rows made 256, one or
+// two, and the SMs with one waited for the others; the y halo comes back per four
+// rows, from L2.  us per reverse step (A and B, every state taped), 16 -> 8 -> 4 rows:
+// 128^2 10.6, 8.3, 7.5; 256^2 12.1, 10.8, 9.5; 512^2 12.4, 10.6, 10.6; 768^2 23.9, 20.4, 19.0; with the
+// recompute beside it at 512^2 17.2, 15.7, 15.3.
+template <typename T, bool PAD>
 struct AdjTile;
 template <>
-struct AdjTile<float> {   // two cells per thread, 512 threads (the padded tile phase needs ~50 registers)
+struct AdjTile<float, false> {
     static constexpr int TX = 64, TY = 16, TYT = 8;
 };
 template <>
-struct AdjTile<double> {  // two cells per thread (register budget)
+struct AdjTile<float, true> {
+    static constexpr int TX = 64, TY = 4, TYT = 2;
+};
+template <bool PAD>
+struct AdjTile<double, PAD> {
     static constexpr int TX = 32, TY = 16, TYT = 8;
 };
 
@@ -208,9 +220,12 @@ struct AdjArgs {
     T r, r5, r25;   // r = (sqrt 5 - 3)/2 of Eq. 20's operator and its powers (padded FP32 tiles)
 };
 
+// Row of tiles of this CTA (grid z continues grid y past its limit of 65535).
+__device__ __forceinline__ int tile_row() { return blockIdx.y + gridDim.y * blockIdx.z; }
+
 // FP64 dL/dT slots of a tile kernel's CTAs: one per warp.
-template <typename T>
-constexpr int adj_warps() { return AdjTile<T>::TX * AdjTile<T>::TYT / 32; }
+template <typename T, bool PAD>
+constexpr int adj_warps() { return AdjTile<T, PAD>::TX * AdjTile<T, PAD>::TYT / 32; }
 
 // Sum of v over each warp (in T), added in FP64 to the warp's own slot
 // cta_slots[w].  Each slot has one writer per launch and the launches are
@@ -296,27 +311,28 @@ __device__ __forceinline__ void store_field(T *base, long long n, long long row,
 constexpr int XO = 28;   // x halo columns staged (>= radius, XO * 4 bytes a multiple of 16)
 constexpr int LO = 4;    // lambda halo columns staged (>= 1)
 
-// HDM derivatives of a padded FP32 tile (64 x 16 cells) of a staged field,
-// written to D[ly * 64 + lx] (along x) and D[1024 + ly * 64 + lx] (along y),
+// HDM derivatives of a padded FP32 tile (64 columns x TY rows) of a staged field,
+// written to D[ly * 64 + lx] (along x) and D[64 TY + ly * 64 + lx] (along y),
 // both radius-26 operators in recurrence form on packed pairs (hdm_window4_paired).
 // Along x, tile row ly is staged at X + ly * XP with tile column c at X + ly *
-// XP + 28 + c; work items 0..255 take four cells of a row each from one
+// XP + 28 + c; the first 16 TY work items take four cells of a row each from one
 // 60-value window of 16-byte loads.  Along y, tile cell (lx, ly) is staged at
-// Y + (26 + ly) * YP + yc0 + lx (26 halo rows on each side); items 256..511
-// take four cells of a column each from one 56-row window.  Thread k of the
-// CTA (at least 512 threads) takes item k; the caller synchronises the CTA
-// before and after.  ABS: the field enters as its magnitude.
+// Y + (26 + ly) * YP + yc0 + lx (26 halo rows on each side); the other 16 TY items
+// take four cells of a column each from one 56-row window.  Thread k of the CTA
+// takes item k; the caller synchronises the CTA before and after.  ABS: the field
+// enters as its magnitude.
 template <bool ABS>
 __device__ __forceinline__ void tile_hdm(const float *X, int XP, const float *Y, int YP, int yc0, float *D,
                                          const Model<float> &m, float r, float r5, float r25) {
     auto mag = [](float v) { return ABS ? fabsf(v) : v; };
     const int item = threadIdx.x + blockDim.x * threadIdx.y;
-    if (item >= 512) return;
+    constexpr int TY = AdjTile<float, true>::TY, NXI = 16 * TY;
+    if (item >= 2 * NXI) return;
     float t[60], d[4];
     float2 tp[28];   // deviations paired about the window's centre (hdm_window4_paired)
 #pragma unroll
     for (int p = 0; p < 60; ++p) t[p] = 0.f;
-    if (item < 256) {
+    if (item < NXI) {
         const int ly = item >> 4, g = item & 15;
         const float *w = X + ly * XP + 4 * g;    // window position p = tile column 4g - 28 + p
 #pragma unroll
@@ -330,7 +346,7 @@ __device__ __forceinline__ void tile_hdm(const float *X, int XP, const float *Y,
         hdm_window4_paired(tp, m.wx[1], m.wx[2], r, r5, r25, d);
         *reinterpret_cast<float4 *>(D + ly * 64 + 4 * g) = make_float4(d[0], d[1], d[2], d[3]);
     } else {
-        const int i = item - 256, cx = i & 63, h = i >> 6;
+        const int i = item - NXI, cx = i & 63, h = i >> 6;
         const float *col = Y + 4 * h * YP + yc0 + cx;   // window position p = staged row 4h - 2 + p
 #pragma unroll
         for (int p = 2; p <= 57; ++p) t[p] = col[(p - 2) * YP];
@@ -339,7 +355,7 @@ __device__ __forceinline__ void tile_hdm(const float *X, int XP, const float *Y,
         for (int j = 0; j < 28; ++j) tp[j] = make_float2(mag(t[2 + j]) - ref, mag(t[57 - j]) - ref);
         hdm_window4_paired(tp, m.wy[1], m.wy[2], r, r5, r25, d);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) D[1024 + (4 * h + c) * 64 + cx] = d[c];
+        for (int c = 0; c < 4; ++c) D[64 * TY + (4 * h + c) * 64 + cx] = d[c];
     }
 }
 
@@ -425,13 +441,15 @@ __device__ __forceinline__ void adj_local(const T (&g)[kQ], T om1, T r, T inv, T
 // stencil field is staged with its halo (element-wise asynchronous copies)
 // and differentiated here.
 template <typename T, bool SC, bool CDM, bool TAU1, int KC>
-__global__ void __launch_bounds__(AdjTile<T>::TX *AdjTile<T>::TYT) adj_a_kernel(const AdjArgs<T> a) {
-    constexpr int TX = AdjTile<T>::TX, TY = AdjTile<T>::TY, TYT = AdjTile<T>::TYT;
+__global__ void __launch_bounds__(AdjTile<T, false>::TX *AdjTile<T, false>::TYT) adj_a_kernel(const AdjArgs<T> a) {
+    using Tl = AdjTile<T, false>;
+    constexpr int TX = Tl::TX, TY = Tl::TY, TYT = Tl::TYT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const Model<T> &m = a.m;
     const int nx = m.nx, ny = m.ny;
     const long long n = (long long)nx * ny;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    const int by = tile_row(), x0 = blockIdx.x * TX, y0 = by * TY;
+    if (y0 >= ny) return;
     const int hx = CDM ? 1 : (KC ? KC : m.kx), hy = CDM ? 1 : (KC ? KC : m.ky);
     // staged field: S[ly * W + hx + lx] = q(x0 + lx, y0 - hy + ly); lambda tile
     // L[(k * LH + ly) * LW + 1 + lx] = lambda_k(x0 + lx, y0 - 1 + ly)
@@ -540,7 +558,7 @@ __global__ void __launch_bounds__(AdjTile<T>::TX *AdjTile<T>::TYT) adj_a_kernel(
             }
         }
     }
-    if (SC) warp_sum_into(tacc, a.Tpart + (size_t)(blockIdx.x + gridDim.x * blockIdx.y) * adj_warps<T>());
+    if (SC) warp_sum_into(tacc, a.Tpart + ((size_t)blockIdx.x + (size_t)gridDim.x * by) * adj_warps<T, false>());
 }
 
 // Kernel A in the padded FP32 layout of the single-pass kernel.  The forward
@@ -553,8 +571,10 @@ __global__ void __launch_bounds__(AdjTile<T>::TX *AdjTile<T>::TYT) adj_a_kernel(
 // stream (ordered by an event); lambda and every write wait for the previous
 // reverse step's kernel B.
 template <bool SC, bool TAU1>
-__global__ void __launch_bounds__(AdjTile<float>::TX *AdjTile<float>::TYT) adj_a_rec_kernel(const AdjArgs<float> a) {
-    constexpr int TX = AdjTile<float>::TX, TY = AdjTile<float>::TY, TYT = AdjTile<float>::TYT, NC = TY / TYT;
+__global__ void __launch_bounds__(AdjTile<float, true>::TX *AdjTile<float, true>::TYT)
+    adj_a_rec_kernel(const AdjArgs<float> a) {
+    using Tl = AdjTile<float, true>;
+    constexpr int TX = Tl::TX, TY = Tl::TY, TYT = Tl::TYT, NC = TY / TYT;
     constexpr int LW = TX + 2 * LO, LH = TY + 2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // lambda tile L[(k * LH + ly) * LW + LO + lx] = lambda_k(x0 + lx, y0 - 1 + ly)
@@ -563,7 +583,8 @@ __global__ void __launch_bounds__(AdjTile<float>::TX *AdjTile<float>::TYT) adj_a
     const Model<float> &m = a.m;
     const int nx = m.nx, ny = m.ny;
     const long long n = (long long)nx * ny;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    const int by = tile_row(), x0 = blockIdx.x * TX, y0 = by * TY;
+    if (y0 >= ny) return;
     const int tid = threadIdx.x + TX * threadIdx.y;
     const int ncore = min(TX, nx - x0);   // a multiple of 4
     const uint32_t lrow = (ncore + 2 * LO) * sizeof(float);
@@ -684,12 +705,13 @@ __global__ void __launch_bounds__(AdjTile<float>::TX *AdjTile<float>::TYT) adj_a
             }
         }
     }
-    if (SC) warp_sum_into(tacc, a.Tpart + (size_t)(blockIdx.x + gridDim.x * blockIdx.y) * adj_warps<float>());
+    if (SC) warp_sum_into(tacc, a.Tpart + ((size_t)blockIdx.x + (size_t)gridDim.x * by) * adj_warps<float, true>());
 }
 
 template <typename T, bool SC, bool CDM, bool TAU1, int KC, bool PAD>
-__global__ void __launch_bounds__(AdjTile<T>::TX *AdjTile<T>::TYT) adj_b_kernel(const AdjArgs<T> a) {
-    constexpr int TX = AdjTile<T>::TX, TY = AdjTile<T>::TY, TYT = AdjTile<T>::TYT;
+__global__ void __launch_bounds__(AdjTile<T, PAD>::TX *AdjTile<T, PAD>::TYT) adj_b_kernel(const AdjArgs<T> a) {
+    using Tl = AdjTile<T, PAD>;
+    constexpr int TX = Tl::TX, TY = Tl::TY, TYT = Tl::TYT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const Model<T> &m = a.m;
     const int nx = m.nx, ny = m.ny;
@@ -705,9 +727,10 @@ __global__ void __launch_bounds__(AdjTile<T>::TX *AdjTile<T>::TYT) adj_b_kernel(
     T *SY = SX + WX * HX;
     uint64_t *bars = reinterpret_cast<uint64_t *>(SY + WY * HY);
     constexpr bool RECUR = PAD && KC == 26 && !CDM;
-    static_assert(!RECUR || TX * TYT >= 512, "the tile phase takes one work item per thread");
+    static_assert(!RECUR || TX * TYT >= 32 * TY, "the tile phase takes one work item per thread");
     T *DT = reinterpret_cast<T *>(bars + 2);   // padded FP32 tiles: D_bar's derivatives over the tile
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    const int by = tile_row(), x0 = blockIdx.x * TX, y0 = by * TY;
+    if (y0 >= ny) return;
     if constexpr (PAD) {
         const int tid = threadIdx.x + TX * threadIdx.y;
         if (tid == 0) {
@@ -812,7 +835,7 @@ __global__ void __launch_bounds__(AdjTile<T>::TX *AdjTile<T>::TYT) adj_b_kernel(
             }
         }
     }
-    warp_sum_into(tacc, a.Tpart + (size_t)(blockIdx.x + gridDim.x * blockIdx.y) * adj_warps<T>());
+    warp_sum_into(tacc, a.Tpart + ((size_t)blockIdx.x + (size_t)gridDim.x * by) * adj_warps<T, PAD>());
 }
 
 // lambda at the final step from dL/drho_T (rho_T = sum_i f_i): lambda_i = g
@@ -888,9 +911,11 @@ int blocks_for(long long n) {
     return (int)(b < 1 ? 1 : (b > 152 * 16 ? 152 * 16 : b));
 }
 
-template <typename T>
+template <typename T, bool PAD>
 dim3 adj_grid(int nx, int ny) {
-    return dim3((nx + AdjTile<T>::TX - 1) / AdjTile<T>::TX, (ny + AdjTile<T>::TY - 1) / AdjTile<T>::TY);
+    using Tl = AdjTile<T, PAD>;
+    const int rows = (ny + Tl::TY - 1) / Tl::TY, y = std::min(rows, 65535);
+    return dim3((nx + Tl::TX - 1) / Tl::TX, y, (rows + y - 1) / y);
 }
 
 // Launch with programmatic stream serialization when `pdl`: the kernel may
@@ -913,7 +938,8 @@ cudaError_t launch_pdl(bool pdl, K kern, dim3 grid, dim3 block, size_t smem, cud
 
 template <typename T, bool SC, bool CDM, bool TAU1, int KC, bool PAD>
 cudaError_t launch_adj_t(const AdjArgs<T> &a, bool overlap_prev, cudaStream_t s) {
-    constexpr int TX = AdjTile<T>::TX, TY = AdjTile<T>::TY, TYT = AdjTile<T>::TYT;
+    using Tl = AdjTile<T, PAD>;
+    constexpr int TX = Tl::TX, TY = Tl::TY, TYT = Tl::TYT;
     const int hx = CDM ? 1 : (KC ? KC : a.m.kx), hy = CDM ? 1 : (KC ? KC : a.m.ky);
     const int XS = PAD ? XO : hx;
     constexpr bool RECUR = PAD && KC == 26 && !CDM;   // B: tile derivatives after the barrier
@@ -946,7 +972,7 @@ cudaError_t launch_adj_t(const AdjArgs<T> &a, bool overlap_prev, cudaStream_t s)
         if (e == cudaSuccess && cache) set_b[dev] = smem_b;
     }
     if (e != cudaSuccess) return e;
-    const dim3 grid = adj_grid<T>(a.m.nx, a.m.ny), block(TX, TYT);
+    const dim3 grid = adj_grid<T, PAD>(a.m.nx, a.m.ny), block(TX, TYT);
     // the padded FP32 kernels wait for their predecessor's output (griddep_wait),
     // so they may overlap it: A with the previous step's B unless an event wait
     // on the recompute's stream precedes it (the first step of a segment), B
@@ -954,7 +980,7 @@ cudaError_t launch_adj_t(const AdjArgs<T> &a, bool overlap_prev, cudaStream_t s)
     e = launch_pdl(PAD && overlap_prev, ka, grid, block, smem_a, s, a);
     if (e != cudaSuccess) return e;
     AdjArgs<T> b = a;
-    b.Tpart = a.Tpart + (size_t)grid.x * grid.y * adj_warps<T>();
+    b.Tpart = a.Tpart + (size_t)grid.x * grid.y * grid.z * adj_warps<T, PAD>();
     e = launch_pdl(PAD, kb, grid, block, smem_b, s, b);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
@@ -981,8 +1007,8 @@ cudaError_t launch_adj_k(const AdjArgs<T> &a, bool padded, bool overlap_prev, cu
 
 template <typename T>
 int adjoint_slots(int nx, int ny) {
-    const dim3 g = adj_grid<T>(nx, ny);
-    return 2 * (int)(g.x * g.y) * adj_warps<T>();
+    const dim3 g = adj_grid<T, false>(nx, ny), p = adj_grid<T, true>(nx, ny);   // (enough for either layout)
+    return 2 * std::max((int)(g.x * g.y * g.z) * adj_warps<T, false>(), (int)(p.x * p.y * p.z) * adj_warps<T, true>());
 }
 
 AdjLayout adjoint_layout(int nx, int ny, bool padded, bool tau1) {
