@@ -70,24 +70,27 @@ lbm_status run_step(const lbm_params &p, const lbm::ModelScalars &ms, const void
     m.aal = (T)ms.aal;
     m.k = (T)ms.k;
     m.omega = (T)(1.0 / p.tau);
-    const int radius = p.hdm_radius ? p.hdm_radius : (p.prec == LBM_F64 ? 40 : 26);
-    double wx[kMaxRadius + 1] = {}, wy[kMaxRadius + 1] = {};
     m.walls = (p.flags & LBM_FLAG_WALLS_Y) ? 1 : 0;
-    const int ny_line = m.walls ? 2 * p.ny : p.ny;   // walls: the mirrored column's period
-    if (lbm_hdm_weights(p.nx, radius, wx, &m.kx) != LBM_OK || lbm_hdm_weights(ny_line, radius, wy, &m.ky) != LBM_OK)
-        return LBM_E_INVALID;
-    for (int j = 0; j <= kMaxRadius; ++j) {
-        m.wx[j] = (T)wx[j];
-        m.wy[j] = (T)wy[j];
+    const bool sc = p.force == LBM_FORCE_SC, cdm = p.grad == LBM_GRAD_CDM;
+    const bool wide = wide_step_supported(p) && (cdm || wide_sums_bytes(p.nx, p.ny) <= kSumsBytes);
+    if (!wide) {   // (the block sums need no weights, which cost more than the launches)
+        const int radius = p.hdm_radius ? p.hdm_radius : (p.prec == LBM_F64 ? 40 : 26);
+        double wx[kMaxRadius + 1] = {}, wy[kMaxRadius + 1] = {};
+        const int ny_line = m.walls ? 2 * p.ny : p.ny;   // walls: the mirrored column's period
+        if (lbm_hdm_weights(p.nx, radius, wx, &m.kx) != LBM_OK || lbm_hdm_weights(ny_line, radius, wy, &m.ky) != LBM_OK)
+            return LBM_E_INVALID;
+        for (int j = 0; j <= kMaxRadius; ++j) {
+            m.wx[j] = (T)wx[j];
+            m.wy[j] = (T)wy[j];
+        }
     }
     cudaStream_t s = (cudaStream_t)p.stream;
     int *err = (int *)scratch;
     m.chk = err;
     T *q = (T *)((unsigned char *)scratch + kErrBytes);
-    const bool sc = p.force == LBM_FORCE_SC, cdm = p.grad == LBM_GRAD_CDM;
     if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) return LBM_E_CUDA;
     cudaError_t e;
-    if (wide_step_supported(p) && (cdm || wide_sums_bytes(p.nx, p.ny) <= kSumsBytes)) {
+    if (wide) {
         e = launch_wide_potential<TS>(m, sc, cdm, (const TS *)f_in, q, (double *)sums, err, s);
         if (e == cudaSuccess)
             e = launch_wide_collide<TS>(m, sc, cdm, (const TS *)f_in, q, (double *)sums, (TS *)f_out, s);
