@@ -97,6 +97,11 @@ lbm_status model_scalars(const lbm_params &p, ModelScalars *s) {
 // and either stream at the higher priority starved the other (11 % slower).
 constexpr int kTapeSlots = 2;
 static_assert(kTapeSlots >= 2, "the recompute runs at least one segment ahead");
+// Records of further segments that the forward keeps where memory allows, so that
+// the sweep need not recompute them: at most this many bytes per context.  144
+// steps at 512^2 (12 segments of 12) need 0.77 GB for all of them; a reverse step
+// costs 10.6 us with its record kept and 15.3 us beside a recompute.
+constexpr size_t kExtraTapeBytes = size_t(4) << 30;
 
 struct lbm_ctx {
     lbm_params p{};
@@ -158,6 +163,9 @@ struct lbm_ctx {
     void *lam[2] = {nullptr, nullptr};
     void *aux = nullptr;
     double *asums = nullptr;          // block sums of D_bar (FP64 block-sum lattices)
+    char *extra = nullptr;            // records and stencil fields of extra_segs more segments
+    int extra_segs = 0;
+    size_t extra_rec = 0, extra_q = 0;   // bytes of a record, of a field there
     double *slots = nullptr;
 };
 
@@ -479,7 +487,10 @@ void free_tape(lbm_ctx *c) {
     c->bw_start = nullptr;
     dev_free(c->aux);
     dev_free(c->asums);
+    dev_free(c->extra);
     dev_free(c->slots);
+    c->extra = nullptr;
+    c->extra_segs = 0;
     c->aux = nullptr;
     c->asums = nullptr;
     c->slots = nullptr;
@@ -535,6 +546,26 @@ template <typename T>
 int tape_slots(const lbm_ctx *c) {
     return tape_wide(c) ? wide_adjoint_slots(c->p.nx, c->p.ny) : adjoint_slots<T>(c->p.nx, c->p.ny);
 }
+
+// Where the records and stencil fields of a segment's states lie: the last two
+// segments' in their slots, those of the segments before them in the extra tape as
+// far as it goes (while it still holds what the forward wrote), the others' in the
+// slot they are recomputed into.
+struct TapeMap {
+    const lbm_ctx *c;
+    int C, K, first;   // K: the last segment; first: the first one whose records the forward keeps
+    TapeMap(const lbm_ctx *c_, int nsteps, int C_, bool taped) : c(c_), C(C_), K((nsteps - 1) / C_) {
+        first = std::max(0, K - 1 - (taped ? std::min(c->extra_segs, std::max(0, K - 1)) : 0));
+    }
+    bool in_extra(int k) const { return k >= first && k < K - 1; }
+    char *extra_segment(int k) const { return c->extra + (size_t)(K - 2 - k) * C * (c->extra_rec + c->extra_q); }
+    void *record(int k, int j) const {
+        return in_extra(k) ? extra_segment(k) + j * c->extra_rec : c->seg[(k % kTapeSlots) * C + j];
+    }
+    void *field(int k, int j) const {
+        return in_extra(k) ? extra_segment(k) + C * c->extra_rec + j * c->extra_q : c->segq[(k % kTapeSlots) * C + j];
+    }
+};
 
 template <typename T>
 lbm_status tape_forward(lbm_ctx *c, const T *rho0, int nsteps, int C, T *rhoT) {
@@ -603,6 +634,20 @@ lbm_status tape_forward(lbm_ctx *c, const T *rho0, int nsteps, int C, T *rhoT) {
                 free_tape(c);
                 return fail(c, LBM_E_NOMEM, "not enough device memory for the reverse sweep buffers");
             }
+            if (tape_rec(c)) {   // (done without if it cannot be had)
+                c->extra_rec = (sbytes + 255) / 256 * 256;
+                c->extra_q = (qbytes + 255) / 256 * 256;
+                const size_t per = (size_t)C * (c->extra_rec + c->extra_q);
+                const int want = (int)std::min<size_t>(std::max(0, (nsteps - 1) / C - 1), kExtraTapeBytes / per);
+                if (want > 0) {
+                    if (dev_alloc(&c->extra, want * per) == cudaSuccess) {
+                        c->extra_segs = want;
+                    } else {
+                        cudaGetLastError();
+                        c->extra = nullptr;
+                    }
+                }
+            }
         }
         c->tape_C = C;
     }
@@ -613,23 +658,24 @@ lbm_status tape_forward(lbm_ctx *c, const T *rho0, int nsteps, int C, T *rhoT) {
     // into their slots, so the sweep starts with no recompute: segment k's
     // stencil fields of states k C .. in slot k % kTapeSlots, and its states
     // k C + 1 .. (contexts with a record: the records of states k C .., the
-    // states themselves staying in the scratch pair).
-    const int K = (nsteps - 1) / C, t0 = K * C, sl = K % kTapeSlots, nseg = C > 1 ? C - 1 : 0;
+    // states themselves staying in the scratch pair), and of the segments before
+    // them into the extra tape as far as it goes.
+    const TapeMap map(c, nsteps, C, true);
+    const int K = map.K, t0 = K * C, sl = K % kTapeSlots, nseg = C > 1 ? C - 1 : 0;
     const int slp = (K + kTapeSlots - 1) % kTapeSlots;   // the slot of segment K - 1
-    const int tp = K >= 1 ? t0 - C : t0;   // the first step of the taped segments
+    const int tp = map.first * C;   // the first step of the taped segments
     auto fbuf = [&](int t) -> void * {   // where state t (>= 1) goes
         if (t % C == 0) return c->ckpt[t / C];
         if (!tape_rec(c) && t > t0 && t < nsteps) return c->seg[sl * nseg + (t - t0 - 1)];
-        if (!tape_rec(c) && t > tp && t < t0) return c->seg[slp * nseg + (t - tp - 1)];
+        if (!tape_rec(c) && t > tp && t < t0) return c->seg[slp * nseg + (t - tp - 1)];   // (no extra tape there)
         return c->tmp[t & 1];
     };
     auto rbuf = [&](int t) -> void * {   // where the record of state t goes
         if (!tape_rec(c) || t < tp) return nullptr;
-        return c->seg[((t / C) % kTapeSlots) * C + t % C];
+        return map.record(t / C, t % C);
     };
     auto qbuf = [&](int t) -> void * {   // the stencil field of state t
-        if (t >= t0 && t < nsteps) return c->segq[sl * C + (t - t0)];
-        if (t >= tp && t < t0) return c->segq[slp * C + (t - tp)];
+        if (t >= tp && t < nsteps) return map.field(t / C, t % C);
         if (tape_fused(c) && t % C == 0) return c->ckptq[t / C];
         return tape_fused(c) ? c->qpad_tape[t & 1] : c->q;
     };
@@ -682,8 +728,10 @@ lbm_status tape_backward(lbm_ctx *c, const T *grad_rhoT, T *grad_rho0, double *g
     // slot sl: states seg[sl * nseg + j], or records seg[sl * C + j], and
     // stencil fields segq[sl * C + j]
     auto segf = [&](int sl, int j) { return c->seg[sl * nseg + j]; };
-    auto segrec = [&](int sl, int j) { return c->seg[sl * C + j]; };
-    auto segqf = [&](int sl, int j) { return c->segq[sl * C + j]; };
+    // the segments that the forward left taped
+    const bool taped = c->tape_last_ready;
+    c->tape_last_ready = false;   // the sweep reuses the slots
+    const TapeMap map(c, N, C, taped);
     // Recompute segment k from its checkpoint with the forward kernels on
     // stream s into slot sl: the stencil field of every state t0 .. t1-1, and
     // the states t0+1 .. t1-1 (with a record: the records of states t0 .. t1-1,
@@ -694,16 +742,16 @@ lbm_status tape_backward(lbm_ctx *c, const T *grad_rhoT, T *grad_rho0, double *g
         cudaError_t r = cudaSuccess;
         if constexpr (std::is_same_v<T, float>) {   // (FP64 contexts never take the single-pass kernel)
             if (tape_fused(c)) {
-                r = cudaMemcpyAsync(segqf(sl, 0), c->ckptq[k], sizeof(float) * (size_t)fused_q_pitch(nx) * ny,
+                r = cudaMemcpyAsync(map.field(k, 0), c->ckptq[k], sizeof(float) * (size_t)fused_q_pitch(nx) * ny,
                                     cudaMemcpyDeviceToDevice, s);
                 const void *cur = c->ckpt[k];
                 for (int t = t0; t < t1 && r == cudaSuccess; ++t) {
                     // (programmatic launches here too: plain ones, which hold no SM
                     // resources while they wait, made the sweep 4 % slower)
                     void *dst = c->tmp[(t + 1) & 1];
-                    void *qn = t + 1 < t1 ? segqf(sl, t + 1 - t0) : c->qpad_tape[0];
-                    r = launch_fused_step(m, is_sc(c), is_cdm(c), (const float *)cur, (const float *)segqf(sl, t - t0),
-                                          (float *)dst, (float *)qn, c->err, rows, s, true, (float *)segrec(sl, t - t0),
+                    void *qn = t + 1 < t1 ? map.field(k, t + 1 - t0) : c->qpad_tape[0];
+                    r = launch_fused_step(m, is_sc(c), is_cdm(c), (const float *)cur, (const float *)map.field(k, t - t0),
+                                          (float *)dst, (float *)qn, c->err, rows, s, true, (float *)map.record(k, t - t0),
                                           (t & 1) != 0);
                     cur = dst;
                 }
@@ -712,14 +760,14 @@ lbm_status tape_backward(lbm_ctx *c, const T *grad_rhoT, T *grad_rho0, double *g
         }
         const void *cur = c->ckpt[k];
         for (int t = t0; t < t1 && r == cudaSuccess; ++t) {
-            r = tape_potential<T>(c, m, cur, segqf(sl, t - t0), s);
+            r = tape_potential<T>(c, m, cur, map.field(k, t - t0), s);
             if (r != cudaSuccess) break;
             if (tape_wide(c)) {   // (the segment's last step too: its record)
                 void *dst = c->tmp[(t + 1) & 1];
-                r = tape_collide<T>(c, m, cur, segqf(sl, t - t0), dst, segrec(sl, t - t0), s);
+                r = tape_collide<T>(c, m, cur, map.field(k, t - t0), dst, map.record(k, t - t0), s);
                 cur = dst;
             } else if (t < t1 - 1) {
-                r = tape_collide<T>(c, m, cur, segqf(sl, t - t0), segf(sl, t - t0), nullptr, s);
+                r = tape_collide<T>(c, m, cur, map.field(k, t - t0), segf(sl, t - t0), nullptr, s);
                 cur = segf(sl, t - t0);
             }
         }
@@ -740,12 +788,9 @@ lbm_status tape_backward(lbm_ctx *c, const T *grad_rhoT, T *grad_rho0, double *g
     const int K = (N - 1) / C;
     for (int j = 0; j < kTapeSlots && e == cudaSuccess; ++j)   // orders rstream after the seed
         e = cudaEventRecord(c->adj_done[j], as);
-    // segments K and K - 1 are left in their slots by the forward
-    const bool taped = c->tape_last_ready;
-    c->tape_last_ready = false;   // the sweep reuses the slots
     auto rec = [&](int j) {
         cudaError_t r = cudaStreamWaitEvent(c->rstream, c->adj_done[j % kTapeSlots], 0);
-        if (r == cudaSuccess && !(taped && j >= K - 1)) r = recompute(j, j % kTapeSlots, c->rstream);
+        if (r == cudaSuccess && !(taped && j >= map.first)) r = recompute(j, j % kTapeSlots, c->rstream);
         if (r == cudaSuccess) r = cudaEventRecord(c->rec_done[j % kTapeSlots], c->rstream);
         return r;
     };
@@ -757,10 +802,10 @@ lbm_status tape_backward(lbm_ctx *c, const T *grad_rhoT, T *grad_rho0, double *g
         if (e == cudaSuccess) e = cudaStreamWaitEvent(as, c->rec_done[sl], 0);
         const int t0 = k * C, t1 = std::min(N, t0 + C);
         for (int t = t1 - 1; t >= t0 && e == cudaSuccess; --t) {
-            const T *ft = (const T *)(tape_rec(c) ? segrec(sl, t - t0) : (t == t0 ? c->ckpt[k] : segf(sl, t - t0 - 1)));
+            const T *ft = (const T *)(tape_rec(c) ? map.record(k, t - t0) : (t == t0 ? c->ckpt[k] : segf(sl, t - t0 - 1)));
             if constexpr (std::is_same_v<T, double>) {
                 if (tape_wide(c)) {
-                    e = launch_wide_adjoint(m, R, aalp, is_sc(c), is_cdm(c), ft, (const double *)segqf(sl, t - t0),
+                    e = launch_wide_adjoint(m, R, aalp, is_sc(c), is_cdm(c), ft, (const double *)map.field(k, t - t0),
                                             (const double *)lam[li], (double *)aux, c->asums, (double *)lam[1 - li], slots,
                                             /*overlap_prev=*/t != t1 - 1, as);
                     li = 1 - li;
@@ -768,7 +813,7 @@ lbm_status tape_backward(lbm_ctx *c, const T *grad_rhoT, T *grad_rho0, double *g
                 }
             }
             e = launch_adjoint_step<T>(m, R, aalp, is_sc(c), is_cdm(c), tau1, tape_fused(c), lay, ft,
-                                       (const T *)segqf(sl, t - t0), qpitch, qoff, (const T *)lam[li], (T *)aux,
+                                       (const T *)map.field(k, t - t0), qpitch, qoff, (const T *)lam[li], (T *)aux,
                                        (T *)lam[1 - li], slots, c->err, /*overlap_prev=*/t != t1 - 1, as);
             li = 1 - li;
         }
