@@ -800,8 +800,10 @@ int fused_q_pitch(int nx) { return nx + 2 * QG; }
 // 126; 4096^2 225, 227, 221 (tau 0.9: 225, 240, 225).  The CDM variant has no column
 // recurrences to start, so short segments cost it little and on large lattices the
 // memory system's tail decides instead: it follows this rule while one wave of at
-// most 9 slabs does (1024^2 19.1 -> 13.5 us), else the one before (2048^2 57.6 us
-// against 58.5 at one wave of 17 slabs).
+// most 9 slabs does (1024^2 19.1 -> 13.5 us), else the one before (2048^2 57.6 us at 126
+// rows against 58.5 at one wave of 17 slabs), with 62 rows for 126 where that makes
+// fewer wave-slabs (2048^2, 306 CTAs of 126 rows for 304 slots: 57.6 -> 54.1 us, tau 0.9
+// 59.8 -> 57.0; 4096^2 keeps 126: 220, at 62 rows 214, tau 0.9 225 and 226).
 int fused_auto_seg_rows(int nx, int ny, int num_sms, bool cdm) {
     const long long strips = (nx + TXI - 1) / TXI, slots = 2LL * num_sms;
     // slabs of the shortest segments that make at most `waves` full waves (0: none do)
@@ -811,9 +813,11 @@ int fused_auto_seg_rows(int nx, int ny, int num_sms, bool cdm) {
         return ((ny + segs - 1) / segs + 2 + SLAB - 1) / SLAB;
     };
     if (cdm && !(slabs_for(1) >= 1 && slabs_for(1) <= 9)) {
+        auto ctas = [&](int h) { return strips * ((ny + h - 1) / h); };
+        auto cost = [&](int h) { return (ctas(h) + slots - 1) / slots * ((h + 2) / SLAB); };
         const int cand[] = {126, 62, 30, 14, 6};
         for (int h : cand)
-            if (strips * ((ny + h - 1) / h) >= num_sms) return h;
+            if (ctas(h) >= num_sms) return h == 126 && cost(62) < cost(126) ? 62 : h;
         return 6;
     }
     long long best = 0, rows = 126;   // (strips alone beyond the waves tried: tall segments)
