@@ -197,4 +197,15 @@ cudaError_t launch_sum_slots(const double *slots, int nslots, double *out, cudaS
 template <typename T>
 cudaError_t launch_density(long long n, const T *f, T *rho, cudaStream_t s);
 
+// Dynamic shared memory that bounds the CTAs of a grid of `tiles` per SM to their
+// even share, for grids of more than half the SMs and up to `most` CTAs per SM; 0
+// otherwise.  A grid that is placed while its predecessor still runs otherwise
+// piles up on the SMs that have room first.  (GB300: 152 SMs of 228 KB, of which a
+// CTA may take 227.)
+constexpr int kSMs = 152, kSMBytes = 228 * 1024;
+inline size_t spread_smem(long long tiles, int most) {
+    const long long per = (tiles + kSMs - 1) / kSMs;
+    return 2 * tiles > kSMs && per <= most ? (size_t)(kSMBytes / (per + 1)) + 1024 : 0;
+}
+
 }  // namespace lbm

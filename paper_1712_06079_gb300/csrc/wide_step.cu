@@ -26,19 +26,26 @@
 // Tiles of 16 x 8 cells, 128 threads, one cell per thread: four warps reach all
 // four FP64 units of an SM, and 128^2 or 1024 x 8 cells still spread over 128
 // or 64 SMs.  For tau = 1 the BGK term vanishes and the equilibrium at u is
-// skipped.  Both passes are launched with programmatic serialization and let
-// the next grid in after their arithmetic: let in at the top, its CTAs pile up
-// on the SMs that still have room (16 of them on one SM) and a grid of 128 CTAs
-// runs on 30 SMs (36.8 us per 128^2 step instead of 13.2).
+// skipped.
+//
+// Both passes are launched with programmatic serialization, so the next grid's
+// CTAs are placed while this grid runs, on the SMs that still have room: let in
+// at the top, a grid of 128 CTAs piled up on about 30 SMs (36.8 us per 128^2
+// step).  Grids of up to four CTAs per SM therefore ask for shared memory that
+// lets no more than their even share onto an SM, and let the next grid in at the
+// top: 9.7 us, against 13.2 when it is let in after the arithmetic without that
+// bound (which larger grids do, and grids of at most half the SMs, which fit
+// beside each other), and 14.4 without programmatic launches.
 //
 // Measured, us per step (direct stencil before -> block sums): FP64 128^2 100 ->
-// 13.2, FP32 1024 x 8 35 -> 10.6; at 1024^2 pass 1 takes 92 and pass 2 159, i.e. 53
+// 9.7, FP32 1024 x 8 35 -> 10.5; at 1024^2 pass 1 takes 92 and pass 2 159, i.e. 53
 // and 92 FP64 instructions at one per 64 cycles and unit, which is the bound
 // there; small lattices are left with the latency of two dependent grids.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 
 #include "lbm_internal.h"
 #include "ptx.cuh"
@@ -62,6 +69,7 @@ struct WideArgs {
     int kbx, kby;            // blocks that cover kReach cells, wherever they start
     int ntx;                 // tiles per row of tiles
     double *ys, *yt, *xs, *xt;   // block sums: ys, yt[by * nx + x]; xs, xt[y * nbx + bx]
+    int early;                   // the next grid is let in at the top (see spread)
     long long nys, nxs;      // entries of each pair
 };
 
@@ -224,6 +232,7 @@ __global__ void __launch_bounds__(NT) wide_potential_kernel(const __grid_constan
     const int x = tx * TX + lx, y = ty * TY + ly;
     const bool valid = x < nx && y < ny;
     const long long c = (long long)y * nx + x;
+    if (A.early) ptx::griddep_launch_dependents();
     ptx::griddep_wait();   // the previous step's pass 2 has written f
     double phi = 0.0;
     if (valid) {
@@ -240,7 +249,7 @@ __global__ void __launch_bounds__(NT) wide_potential_kernel(const __grid_constan
         phi = sc ? sqrt(fabs(U)) : U;
         q[c] = sc ? copysign(phi, U) : U;   // s Phi (Eq. 21), s the sign of U, or U (Eq. 8)
     }
-    ptx::griddep_launch_dependents();
+    if (!A.early) ptx::griddep_launch_dependents();
     if (!HDM) return;
     S[ly][lx] = phi;
     __syncthreads();
@@ -266,6 +275,7 @@ __global__ void __launch_bounds__(NT) wide_collide_kernel(const __grid_constant_
     const int x = x0 + lx, y = y0 + ly;
     const bool valid = x < nx && y < ny;
     const long long c = (long long)min(y, ny - 1) * nx + min(x, nx - 1);
+    if (A.early) ptx::griddep_launch_dependents();
     ptx::griddep_wait();   // pass 1 has written q and the block sums
 
     // the rows and columns of the tile's halo: periodic, or mirrored across a wall
@@ -290,7 +300,7 @@ __global__ void __launch_bounds__(NT) wide_collide_kernel(const __grid_constant_
     const double jx = east - west, jy = (fi[2] + fi[5] + fi[6]) - (fi[4] + fi[7] + fi[8]);
     const double inv = 1.0 / r;
     if (HDM) __syncthreads();
-    ptx::griddep_launch_dependents();
+    if (!A.early) ptx::griddep_launch_dependents();
     if (!valid) return;
 
     const double *p = &Q[ly + 1][lx + 1];
@@ -454,6 +464,7 @@ __global__ void __launch_bounds__(NT) wide_adj_a_kernel(const __grid_constant__ 
     const bool valid = x < nx && y < ny;
     const int xc = min(x, nx - 1), yc = min(y, ny - 1);
     const long long c = (long long)yc * nx + xc;
+    if (A.early) ptx::griddep_launch_dependents();
     ptx::griddep_wait();
     auto rec = [&](int k) { return in_bounds(k * n + c, 5 * n, m.chk) ? a.rec[k * n + c] : 1.0; };
     const double r = rec(0), jx = rec(1), jy = rec(2), Dx = rec(3), Dy = rec(4);
@@ -551,7 +562,7 @@ __global__ void __launch_bounds__(NT) wide_adj_a_kernel(const __grid_constant__ 
         SY[ly][lx] = valid ? Dby : 0.0;
         __syncthreads();
     }
-    ptx::griddep_launch_dependents();
+    if (!A.early) ptx::griddep_launch_dependents();
     if (valid) {
         const double v[7] = {Dbx, Dby, rb, kappa, theta, jbx, jby};
 #pragma unroll
@@ -579,6 +590,7 @@ __global__ void __launch_bounds__(NT) wide_adj_b_kernel(const __grid_constant__ 
     const bool valid = x < nx && y < ny;
     const int xc = min(x, nx - 1), yc = min(y, ny - 1);
     const long long c = (long long)yc * nx + xc;
+    if (A.early) ptx::griddep_launch_dependents();
     ptx::griddep_wait();   // A's output
     for (int k = threadIdx.x; k < (TY + 2) * (TX + 2); k += NT) {
         const int ry = k / (TX + 2), rx = k - ry * (TX + 2);
@@ -595,7 +607,7 @@ __global__ void __launch_bounds__(NT) wide_adj_b_kernel(const __grid_constant__ 
         tile_step<false>(A, tx, ty, carry, QY, QX, M);
         __syncthreads();
     }
-    ptx::griddep_launch_dependents();
+    if (!A.early) ptx::griddep_launch_dependents();
     const double *px = &QX[ly + 1][lx + 1], *py = &QY[ly + 1][lx + 1];
     constexpr int QW = TX + 2;
     double dd;   // Dx[D_bar_x] + Dy[D_bar_y]
@@ -648,6 +660,8 @@ int cover(int n, bool mirror) {
     return worst;
 }
 
+constexpr int kSpread = 4;   // CTAs per SM up to which a grid is spread (see the head of the file)
+
 WideArgs args_of(const Model<double> &m, double *sums) {
     WideArgs a{};
     a.m = m;
@@ -669,7 +683,23 @@ WideArgs args_of(const Model<double> &m, double *sums) {
     a.yt = a.ys + a.nys;
     a.xs = a.yt + a.nys;
     a.xt = a.xs + a.nxs;
+    a.early = spread_smem((long long)a.ntx * a.nby, kSpread) > 0;
     return a;
+}
+
+// The dynamic shared-memory limit of a kernel (spread_smem asks for at most half an
+// SM), raised once per kernel and device.
+cudaError_t allow_smem(const void *kern, int dev) {
+    constexpr int kSpreadMax = kSMBytes / 2 + 1024;
+    static std::mutex lock;
+    static struct { const void *kern; int dev; } done[256];   // (a full table sets the limit again)
+    static int n = 0;
+    std::lock_guard<std::mutex> hold(lock);
+    for (int i = 0; i < n; i++)
+        if (done[i].kern == kern && done[i].dev == dev) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpreadMax);
+    if (e == cudaSuccess && n < 256) done[n++] = {kern, dev};
+    return e;
 }
 
 template <typename K, typename... Args>
@@ -678,6 +708,13 @@ cudaError_t launch_grid(K kern, const WideArgs &w, bool pdl, cudaStream_t s, Arg
     cfg.gridDim = dim3((unsigned)((long long)w.ntx * w.nby));
     cfg.blockDim = dim3(NT);
     cfg.stream = s;
+    cfg.dynamicSmemBytes = spread_smem((long long)w.ntx * w.nby, kSpread);
+    if (cfg.dynamicSmemBytes > 0) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = allow_smem((const void *)kern, dev);
+        if (e != cudaSuccess) return e;
+    }
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;

@@ -105,3 +105,25 @@ def test_reverse_step_is_the_complex_step_derivative(nx, ny, eos, force, grad, t
     d = xi[2] - 0.5
     _, dd = oracle.tangent(op, rho0, 5, drho0=d)
     assert abs((grad0 * d).sum() - (v * dd).sum()) < 1e-11 * np.abs(v * dd).sum()
+
+
+@pytest.mark.parametrize("nx,ny", [(608, 16), (616, 16), (304, 256), (304, 264)])
+@pytest.mark.parametrize("prec,tau", [("f64", 1.0), ("f32", 0.9)])
+def test_overlapping_launches_change_nothing(nx, ny, prec, tau):
+    # 76 | 78 tiles and 608 | 627: both sides of the two lines at which the
+    # launches change between spreading over the SMs and not.  Steps whose
+    # launches overlap are bit for bit the steps that are waited for one by one
+    gp, op, _ = make(nx, ny, prec, tau=tau)
+    g, l, _ = oracle.maxwell(op)
+    y, x = np.mgrid[0:ny, 0:nx]
+    wave = np.sin(2 * np.pi * x / nx) * np.cos(2 * np.pi * y / ny)
+    f0 = oracle.init(op, 0.5 * (g + l) + 0.1 * (l - g) * wave, 0.01 * wave, -0.01 * wave)
+    out = []
+    for chunks in ([1] * 8, [8]):
+        with lbm.Lattice(gp) as lat:
+            lat.set_f(f0)
+            for n in chunks:
+                lat.step(n)
+                last = lat.get_f()
+            out.append(last)
+    assert np.isfinite(out[0]).all() and np.array_equal(out[0], out[1])
