@@ -66,7 +66,7 @@ namespace {
 // two, and the SMs with one waited for the others; the y halo comes back per four
 // rows, from L2.  us per reverse step (A and B, every state taped), 16 -> 8 -> 4 rows:
 // 128^2 10.6, 8.3, 7.5; 256^2 12.1, 10.8, 9.5; 512^2 12.4, 10.6, 10.6; 768^2 23.9, 20.4, 19.0; with the
-// recompute beside it at 512^2 17.2, 15.7, 15.3.
+// recompute beside it at 512^2 17.2, 15.7, 15.3 (all before the launches were spread, see launch_adj_t).
 template <typename T, bool PAD>
 struct AdjTile;
 template <>
@@ -946,11 +946,17 @@ cudaError_t launch_adj_t(const AdjArgs<T> &a, bool overlap_prev, cudaStream_t s)
     const size_t dt = RECUR ? 2 * sizeof(T) * TX * TY : 0;
     // A: in the padded layout the lambda tile (tau = 1) and its barrier; else
     // the field with its halo and the lambda tile
-    const size_t smem_a = PAD ? (TAU1 ? sizeof(T) * 3 * (TX + 2 * LO) * (TY + 2) + sizeof(uint64_t) : 0)
+    // Launches that overlap their predecessor (PAD): up to eight CTAs per SM they are
+    // spread over the SMs.  us per reverse step, without -> with: 144^2 7.8 -> 7.2, 256^2
+    // 9.7 -> 7.7, 512^2 10.7 -> 10.0, 700 x 300 11.0 -> 9.9; at nine (640 x 512) 13.1 both,
+    // at ten (600^2) 13.7 -> 14.3, so those go without.
+    const size_t spread = PAD ? spread_smem((long long)((a.m.nx + TX - 1) / TX) * ((a.m.ny + TY - 1) / TY), 8) : 0;
+    const size_t need_a = PAD ? (TAU1 ? sizeof(T) * 3 * (TX + 2 * LO) * (TY + 2) + sizeof(uint64_t) : 0)
                               : sizeof(T) * ((size_t)(TX + 2 * hx) * (TY + 2 * hy) + (TAU1 ? 3 * (TX + 2) * (TY + 2) : 0));
-    const size_t smem_b = (CDM ? sizeof(T) * 2 * (size_t)(TX + 2) * (TY + 2)
+    const size_t need_b = (CDM ? sizeof(T) * 2 * (size_t)(TX + 2) * (TY + 2)
                                : sizeof(T) * ((size_t)(TX + 2 * XS) * TY + (size_t)TX * (TY + 2 * hy))) +
                           (PAD ? 2 * sizeof(uint64_t) : 0) + dt;
+    const size_t smem_a = std::max(need_a, spread), smem_b = std::max(need_b, spread);
     void (*ka)(const AdjArgs<T>) = nullptr;
     if constexpr (PAD) ka = adj_a_rec_kernel<SC, TAU1>;   // T = float
     else ka = adj_a_kernel<T, SC, CDM, TAU1, KC>;

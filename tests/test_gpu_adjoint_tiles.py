@@ -33,3 +33,27 @@ def test_fp32_gradient_follows_fp64(nx, ny, force, tau):
     (ga, fa), (gb, fb) = out["f64"], out["f32"]
     assert np.max(np.abs(fb - fa)) < 1e-4 * np.max(np.abs(fa))
     assert abs(gb - ga) < 2e-3 * abs(ga) + 1e-3
+
+
+@pytest.mark.parametrize("nx,ny", [(128, 152), (132, 152), (512, 608), (516, 608)])
+def test_overlapping_launches_change_nothing(nx, ny):
+    # 76 | 114 tiles and 1216 | 1368: both sides of the lines at which the launches are
+    # spread over the SMs.  A tape with every state and one of short segments, whose first
+    # launches do not overlap, take the same steps: bit for bit the same gradient
+    torch = pytest.importorskip("torch")
+    t = inputs.EOS_TABLE["cs"]
+    xi = inputs.uniform01(nx + 5 * ny, 2 * nx * ny).reshape(2, ny, nx)
+    p = lbm.Params(nx=nx, ny=ny, eos="cs", a=t["a"], b=t["b"], Tr=0.85, k=t["k"], prec="f32",
+                   stream=torch.cuda.current_stream().cuda_stream)
+    g, l = lbm.maxwell(p)
+    x = torch.tensor(inputs.droplet(nx, ny, ny / 4, g, l, 3.0) * (1 + 0.01 * (xi[0] - 0.5)), dtype=torch.float32, device="cuda")
+    v = torch.tensor(xi[1] - 0.5, dtype=torch.float32, device="cuda")
+    out = []
+    for chunk in (1, 9):
+        rT, g0 = torch.empty_like(x), torch.empty_like(x)
+        torch.cuda.synchronize()
+        with lbm.Lattice(p) as lat:
+            lat.adjoint_forward(x.data_ptr(), 9, chunk, rT.data_ptr())
+            lat.adjoint_backward(v.data_ptr(), g0.data_ptr())
+            out.append(g0.cpu().numpy())
+    assert np.isfinite(out[0]).all() and np.array_equal(out[0], out[1])
