@@ -963,19 +963,21 @@ cudaError_t launch_adj_t(const AdjArgs<T> &a, bool overlap_prev, cudaStream_t s)
     auto kb = adj_b_kernel<T, SC, CDM, TAU1, KC, PAD>;
     // the shared-memory limits, set once per device and size (a driver call per
     // launch otherwise); the largest size set so far covers every smaller one
+    const size_t lim_a = PAD ? std::max<size_t>(smem_a, kSpreadMax) : smem_a;
+    const size_t lim_b = PAD ? std::max<size_t>(smem_b, kSpreadMax) : smem_b;
     constexpr int kDevs = 64;
     static size_t set_a[kDevs] = {}, set_b[kDevs] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     const bool cache = dev >= 0 && dev < kDevs;
-    if (!cache || smem_a > set_a[dev]) {
-        e = cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_a);
-        if (e == cudaSuccess && cache) set_a[dev] = smem_a;
+    if (!cache || lim_a > set_a[dev]) {
+        e = cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim_a);
+        if (e == cudaSuccess && cache) set_a[dev] = lim_a;
     }
-    if (e == cudaSuccess && (!cache || smem_b > set_b[dev])) {
-        e = cudaFuncSetAttribute(kb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b);
-        if (e == cudaSuccess && cache) set_b[dev] = smem_b;
+    if (e == cudaSuccess && (!cache || lim_b > set_b[dev])) {
+        e = cudaFuncSetAttribute(kb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim_b);
+        if (e == cudaSuccess && cache) set_b[dev] = lim_b;
     }
     if (e != cudaSuccess) return e;
     const dim3 grid = adj_grid<T, PAD>(a.m.nx, a.m.ny), block(TX, TYT);

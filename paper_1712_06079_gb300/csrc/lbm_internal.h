@@ -202,7 +202,9 @@ cudaError_t launch_density(long long n, const T *f, T *rho, cudaStream_t s);
 // otherwise.  A grid that is placed while its predecessor still runs otherwise
 // piles up on the SMs that have room first.  (GB300: 152 SMs of 228 KB, of which a
 // CTA may take 227.)
-constexpr int kSMs = 152, kSMBytes = 228 * 1024;
+// Kernels launched this way are always given the one limit kSpreadMax, which covers
+// every size, so that threads launching other grids cannot lower it in between.
+constexpr int kSMs = 152, kSMBytes = 228 * 1024, kSpreadMax = kSMBytes / 2 + 1024;
 inline size_t spread_smem(long long tiles, int most) {
     const long long per = (tiles + kSMs - 1) / kSMs;
     return 2 * tiles > kSMs && per <= most ? (size_t)(kSMBytes / (per + 1)) + 1024 : 0;

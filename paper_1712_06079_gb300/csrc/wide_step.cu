@@ -45,7 +45,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 
 #include "lbm_internal.h"
 #include "ptx.cuh"
@@ -687,21 +686,6 @@ WideArgs args_of(const Model<double> &m, double *sums) {
     return a;
 }
 
-// The dynamic shared-memory limit of a kernel (spread_smem asks for at most half an
-// SM), raised once per kernel and device.
-cudaError_t allow_smem(const void *kern, int dev) {
-    constexpr int kSpreadMax = kSMBytes / 2 + 1024;
-    static std::mutex lock;
-    static struct { const void *kern; int dev; } done[256];   // (a full table sets the limit again)
-    static int n = 0;
-    std::lock_guard<std::mutex> hold(lock);
-    for (int i = 0; i < n; i++)
-        if (done[i].kern == kern && done[i].dev == dev) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpreadMax);
-    if (e == cudaSuccess && n < 256) done[n++] = {kern, dev};
-    return e;
-}
-
 template <typename K, typename... Args>
 cudaError_t launch_grid(K kern, const WideArgs &w, bool pdl, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
@@ -710,9 +694,7 @@ cudaError_t launch_grid(K kern, const WideArgs &w, bool pdl, cudaStream_t s, Arg
     cfg.stream = s;
     cfg.dynamicSmemBytes = spread_smem((long long)w.ntx * w.nby, kSpread);
     if (cfg.dynamicSmemBytes > 0) {
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = allow_smem((const void *)kern, dev);
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpreadMax);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchAttribute attr[1];
