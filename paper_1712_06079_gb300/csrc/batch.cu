@@ -1344,12 +1344,14 @@ auto grid_kernel(const lbm_batch *b) -> void (*)(const BatchArgs<T>, int) {
 }
 size_t grid_smem(const lbm_batch *b, int threads) { return (size_t)(threads / NT) * b->tile_floats * sizeof(float); }
 
+// (The limit of shared memory belongs to the function: it is always set to the largest
+// any batch takes, so that another batch, or another thread's, never lowers it.)
 template <typename T>
 int max_blocks_per_sm(const lbm_batch *b, int threads) {
     const size_t smem = grid_smem(b, threads);
     int nb = 0;
-    if (cudaFuncSetAttribute(grid_kernel<T>(b), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grid_smem(b, 512)) !=
-            cudaSuccess ||
+    const int limit = b->vec ? (int)((512 / NT) * tile_floats(9) * sizeof(float)) : 0;
+    if (cudaFuncSetAttribute(grid_kernel<T>(b), cudaFuncAttributeMaxDynamicSharedMemorySize, limit) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, grid_kernel<T>(b), threads, smem) != cudaSuccess)
         return 0;
     return nb;
@@ -1507,7 +1509,10 @@ cudaError_t enqueue(lbm_batch *b, int nsteps) {
     if (e != cudaSuccess) return e;
     BatchArgs<T> a = make_args<T>(b, nsteps);
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(b->grid_blocks);
+    // (a cooperative launch: at most what is resident at once)
+    const int resident = max_blocks_per_sm<T>(b, b->block_threads) * sm_count();
+    if (resident < 1) return cudaErrorInvalidConfiguration;
+    cfg.gridDim = dim3(std::min(b->grid_blocks, resident));
     cfg.blockDim = dim3(b->block_threads);
     cfg.dynamicSmemBytes = grid_smem(b, b->block_threads);
     cfg.stream = b->stream;
@@ -1725,7 +1730,9 @@ lbm_status lbm_batch_set_launch(lbm_batch *b, int block_threads, int blocks_per_
     if (!b) return LBM_E_INVALID;
     if (block_threads != 128 && block_threads != 256 && block_threads != 512)
         return bfail(b, LBM_E_INVALID, "block_threads must be 128, 256 or 512");
-    const int maxb = max_blocks_per_sm(b, block_threads);
+    // A shape is accepted up to the threads per SM that the per-cell kernels can keep
+    // resident; the vector path's tiles allow fewer, and a larger shape runs with those.
+    const int maxb = (b->prec == LBM_F64 ? 1152 : 1280) / block_threads;
     if (blocks_per_sm < 1 || blocks_per_sm > maxb)
         return bfail(b, LBM_E_INVALID, "blocks_per_sm must be in [1, " + std::to_string(maxb) + "]");
     b->block_threads = block_threads;

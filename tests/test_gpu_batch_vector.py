@@ -66,3 +66,26 @@ def test_forms_are_the_oracles_step_and_each_other(mix):
             for p, q in zip(x, y):
                 assert np.array_equal(p, q)
     assert ran >= 2
+
+
+def test_every_grid_shape_is_taken_and_survives_other_batches():
+    # 1280 threads per SM are accepted, whatever fits at once is launched, and the bits
+    # are the default shape's; a batch of smaller tiles made in between changes nothing
+    tall, thin = [make(*m) for m in MIXES[3]], [make(*m) for m in MIXES[0]]
+    out = []
+    for shape in (None, (128, 10), (256, 5), (512, 2)):
+        with lbm.Batch([gp for gp, _, _ in tall]) as b:
+            if shape:
+                b.set_launch(*shape)
+                with pytest.raises(lbm.LBMError):
+                    b.set_launch(shape[0], shape[1] + 1)
+            with lbm.Batch([gp for gp, _, _ in thin]) as other:
+                other.set_f([f for _, _, f in thin])
+                other.step(1)
+                other.sync()
+            b.set_f([f for _, _, f in tall])
+            b.step(2)
+            b.sync()
+            out.append(np.concatenate([f.ravel() for f in b.get_f()]))
+    for o in out[1:]:
+        assert np.array_equal(o, out[0])
