@@ -18,16 +18,17 @@
 // on each side), a group of 128 threads a tile of 64 x 8 cells (lattices of at
 // most 8 rows) or 32 x 16.  The tile's populations are copied into shared memory
 // once per step (cp.async, at the step's start) and serve both phases when every
-// group has one tile; phase B stages the field with its halo, takes d/dx of the
-// four cells from one 60-value window in recurrence form on packed pairs
+// group has one tile; with several, phase B starts with the one that phase A ended
+// with.  Phase B stages the field with its halo, takes d/dx of the four cells from one 60-value window in recurrence form on packed pairs
 // (hdm_window4_paired, as the single-pass kernel does), d/dy likewise from windows
 // of the columns or, on short columns, from the folded weights, and collides the
 // four cells as two packed pairs.  Every other batch (FP64, or with a CDM lattice,
 // another radius or a narrower row in it) takes the form this replaced: one cell a
 // thread, 26 + 26 (40 + 40) taps loaded one by one.  us per step, per-cell form ->
-// vector path: twenty 200^2 lattices in the grid form 86.9 -> 34.9 (two grid
-// barriers with their phases' latency are 9 of it, about 1900 instructions per
-// thread and step the rest); the 64-lattice sweep (590,000 cells) 41.5 -> 26.4 in the
+// vector path: twenty 200^2 lattices in the grid form 86.9 -> 31.6 (34.8
+// before phase B kept the last tile and the barriers lost two fences; waiting per
+// lattice and per group instead of for the whole grid was no faster, 31.7; about 1900
+// instructions per thread and step); the 64-lattice sweep (590,000 cells) 41.5 -> 25.9 in the
 // grid form, 31.8 -> 20.8 with one cluster size, 27.6 -> 18.3 as tuned (grouped).
 //
 // A cell's operations depend on its absolute position only (the groups of four
@@ -100,13 +101,14 @@ __device__ __forceinline__ unsigned long long gtimer() {
 
 // Grid-wide barrier with a wall-time bound: the arrivals of all barriers of the
 // launch are counted in one word, so an arrival needs no answer and a wait polls
-// for `target` arrivals.  Returns false if the batch was aborted (by a timeout
-// here or elsewhere).
+// for `target` arrivals.  The CTA's barrier orders its threads' writes before thread
+// 0's release, and that release before another CTA's acquire and barrier: there is no
+// further fence.  Returns false if the batch was aborted
+// (by a timeout here or elsewhere).
 __device__ bool grid_sync(BarrierState *b, unsigned int target, int *err, unsigned long long limit_ns) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&b->count) : "memory");
         auto arrived = [&] {
             unsigned int v;
@@ -124,7 +126,6 @@ __device__ bool grid_sync(BarrierState *b, unsigned int target, int *err, unsign
                 break;
             }
         }
-        __threadfence();
         ok = !*vabort;
     }
     __syncthreads();
@@ -664,7 +665,7 @@ __global__ void __launch_bounds__(512, 2) batch_kernel(const BatchArgs<T> a, int
     float *S = reinterpret_cast<float *>(smem_raw) + (size_t)g * floats;
     const unsigned int nblocks = gridDim.x;
     const int first = g * (int)nblocks + (int)blockIdx.x, stride = (int)nblocks * (blockDim.x / NT);
-    const bool one = first + stride >= a.ntiles;   // this group has one tile at most: its populations stay for phase B
+    const int last = first + (a.ntiles - 1 - first) / stride * stride;   // its populations stay for phase B, which goes backwards
     unsigned int target = 0;
     for (int step = 0; step < a.nsteps; ++step) {
         const bool odd = ((a.parity0 + step) & 1) != 0;  // (a select, not a dynamic index into the parameters)
@@ -685,12 +686,12 @@ __global__ void __launch_bounds__(512, 2) batch_kernel(const BatchArgs<T> a, int
         }
         if (step == 0 && (int)blockIdx.x == a.skip_block) return;  // test hook: never arrive
         if (!grid_sync(a.bar, target += nblocks, a.err, a.limit_ns)) return;
-        for (int k = first; k < a.ntiles; k += stride) {
+        for (int k = first < a.ntiles ? last : -1; k >= 0; k -= stride) {
             const int4 tile = a.tiles[k];
             const Inst<T> &I = a.inst[tile.x];
             if constexpr (VEC) {
                 const bool thin = I.m.ny <= 8;
-                if (!one) {
+                if (k != last) {
                     if (thin) tile_load<true>(a, f, I, tile, S, t);
                     else tile_load<false>(a, f, I, tile, S, t);
                 }
