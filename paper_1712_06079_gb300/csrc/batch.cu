@@ -25,10 +25,10 @@
 // four cells as two packed pairs.  Every other batch (FP64, or with a CDM lattice,
 // another radius or a narrower row in it) takes the form this replaced: one cell a
 // thread, 26 + 26 (40 + 40) taps loaded one by one.  us per step, per-cell form ->
-// vector path: twenty 200^2 lattices in the grid form 86.9 -> 31.6 (34.8
-// before phase B kept the last tile and the barriers lost two fences; waiting per
-// lattice and per group instead of for the whole grid was no faster, 31.7; about 1900
-// instructions per thread and step); the 64-lattice sweep (590,000 cells) 41.5 -> 25.9 in the
+// vector path: twenty 200^2 lattices in the grid form 86.9 -> 28.4 (waiting per
+// lattice and per group instead of for the whole grid was no faster, and neither was
+// starting the next tile's copy as soon as this one's populations are in registers; about
+// 1900 instructions per thread and step); the 64-lattice sweep (590,000 cells) 41.5 -> 23 in the
 // grid form, 31.8 -> 20.8 with one cluster size, 27.6 -> 18.3 as tuned (grouped).
 //
 // A cell's operations depend on its absolute position only (the groups of four
@@ -658,8 +658,12 @@ __device__ __forceinline__ void cell_collide(const BatchArgs<T> &a, const T *f, 
 }
 
 // Persistent kernel of the grid form; VEC: a batch on the vector path.
+// Registers: shared memory lets three blocks of 256 threads of the vector path onto an
+// SM, so they may take 80 (at 64 it spilled 450 bytes: twenty 200^2 lattices 31.6 -> 28.4
+// us per step, the 64-lattice sweep 25.9 -> 23); the per-cell path keeps 1280 (FP32) or
+// 1152 (FP64) threads resident.
 template <typename T, bool VEC>
-__global__ void __launch_bounds__(512, 2) batch_kernel(const BatchArgs<T> a, int floats) {
+__global__ void __maxnreg__(VEC ? 80 : (sizeof(T) == 4 ? 48 : 56)) batch_kernel(const BatchArgs<T> a, int floats) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int g = threadIdx.x / NT, t = threadIdx.x & (NT - 1);
     float *S = reinterpret_cast<float *>(smem_raw) + (size_t)g * floats;
