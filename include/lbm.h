@@ -237,7 +237,11 @@ lbm_status lbm_gradient(lbm_ctx *c, const double *q, double h, double *gx, doubl
  *   nsteps steps (Eq. 1), density of the final state into the device array
  *   rho_T; the state every checkpoint_interval steps is kept on the device
  *   (checkpoint_interval = ceil(sqrt(nsteps)) gives sqrt(N) checkpointing, 1
- *   keeps every state).  The context is left on the final state.
+ *   keeps every state).  Where a context records states for the reverse step
+ *   (single-pass HDM lattices, FP64 lattices at the default radius), the records
+ *   of further segments are kept as well, up to 4 GiB and half of the free
+ *   memory, so that fewer segments are recomputed; without that memory it does
+ *   with less.  The context is left on the final state.
  * lbm_adjoint_backward: from dL/drho_T (device array) writes dL/drho0 (device
  *   array) and dL/dT, dL/d(T/Tc), dL/dG (host doubles, each may be NULL),
  *   recomputing the states between checkpoints with the same kernels and
@@ -411,13 +415,13 @@ void lbm_batch_destroy(lbm_batch *b);
  *          state at t+1.  Both stay owned by the caller.
  * The step is lbm_step's two-pass form (for LBM_F32: FP32 distributions,
  * FP64 arithmetic).  Its potential field (FP64 in both precisions) and the
- * error word live in one file-scope device array of LBM_STATIC_SCRATCH_BYTES
- * (4 MiB) that every GPU loading the library holds until the process exits,
- * so nx*ny may be at most (4 MiB - 256 B) / 8 = 524,256 cells; larger
+ * error word live in a file-scope device array of LBM_STATIC_SCRATCH_BYTES
+ * (4 MiB), the HDM's block sums in a second one (3 MiB); every GPU loading the
+ * library holds both until the process exits, so nx*ny may be at most (4 MiB - 256 B) / 8 = 524,256 cells; larger
  * lattices are rejected with LBM_E_INVALID before any device work.  The first call on a
- * device looks the array's device address up (with that device current), so
+ * device looks the arrays' device addresses up (with that device current), so
  * make the first call before any stream capture.  Every call, on any stream,
- * shares the one array and leaves its contents behind; the error word is
+ * shares the arrays and leaves their contents behind; the error word is
  * cleared at the start of each call.  Calls whose work overlaps on the GPU
  * therefore race and must be serialised by the caller.  Synchronising:
  * returns LBM_E_UNSTABLE if the step saw a NaN or rho <= 0, LBM_E_CUDA on a

@@ -16,9 +16,9 @@
 // (half-way bounce-back), the same reading as the two-pass kernels.
 //
 // Decomposition.  A CTA of 8 warps owns a strip of TXI = 120 columns and a
-// segment of up to seg_h rows (a launch parameter: by default the tallest of
-// 126, 62, 30, 14, 6 that gives every SM a CTA; the library's tuner times the
-// heights on the live state).  It sweeps the segment in slabs of 8 rows, one
+// segment of up to seg_h rows (a launch parameter: by default the height with
+// the fewest waves x slabs, see fused_auto_seg_rows; the library's tuner times
+// the heights on the live state).  It sweeps the segment in slabs of 8 rows, one
 // warp per row and one lane per 4 consecutive cells.  Lanes 1..30 hold the
 // strip's columns; lanes 0 and 31 hold the 4-column groups just outside it,
 // whose collision is recomputed so that the density at t+1 of every strip

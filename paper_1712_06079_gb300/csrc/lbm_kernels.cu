@@ -1,4 +1,8 @@
-// Two-pass D2Q9 HDM pseudopotential step for sm_103a (FP32 and FP64).
+// Two-pass D2Q9 HDM pseudopotential step for sm_103a (FP32 and FP64) with the
+// direct stencil: lattices with a requested HDM radius, lattices one cell wide and
+// FP32 arithmetic off the single-pass kernel.  (wide_step.cu takes the other
+// lattices, and the FP64 reverse mode, with the same operator as block sums.)
+// Also the gradient of a caller's field, initialisation and the reductions.
 //
 // Pass 1 (potential_kernel): one thread per cell reads the nine SoA
 // distributions (coalesced along x), forms rho (Eq. 3) and writes the
