@@ -29,7 +29,7 @@
 // lattice and per group instead of for the whole grid was no faster, and neither was
 // starting the next tile's copy as soon as this one's populations are in registers; about
 // 1900 instructions per thread and step); the 64-lattice sweep (590,000 cells) 41.5 -> 23 in the
-// grid form, 31.8 -> 20.8 with one cluster size, 27.6 -> 18.3 as tuned (grouped).
+// grid form, 31.8 -> 20.8 with one cluster size, 27.6 -> 16.9 as tuned (grouped).
 //
 // A cell's operations depend on its absolute position only (the groups of four
 // start at multiples of four), packed pairs round as single operations do, and
@@ -1002,8 +1002,8 @@ __device__ __forceinline__ void cluster_vec_steps(const ClusterArgs<float> &a, c
     }
 }
 
-template <int MAXT>
-__global__ void __launch_bounds__(MAXT, 1024 / MAXT) cluster_vec_kernel(const ClusterArgs<float> a) {
+template <int MAXT, int PER>
+__global__ void __launch_bounds__(MAXT, PER) cluster_vec_kernel(const ClusterArgs<float> a) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1395,9 +1395,12 @@ size_t cluster_smem_bytes(const lbm_batch *b, int cluster) {
 // Launch of the cluster form over the instances picked by `in`: kernel, threads
 // per CTA and shared memory.  The vector path's kernel takes a thread per group of
 // four cells of its widest slice whatever `threads` asks (a slice that
-// cluster_smem_bytes admits has at most 851 of them, and never more shared memory
-// than that); up to 512 threads two CTAs share an SM, which with 64 registers and a
-// few spills measured 18.8 us per sweep step against 21.1 with one CTA of 118 registers.
+// cluster_smem_bytes admits has at most 768 of them, and never more shared memory than
+// that).  Up to 512 threads two CTAs share an SM, which with 64 registers and 650 bytes
+// of spills measured 18.8 us per step of the 64-lattice sweep (one cluster size) against
+// 21.1 with one CTA of 118 registers.  Above that there is one CTA per SM in any case and
+// it may take 80 registers: as tuned, 34 + 12 of the 64 lattices in CTAs of 744 threads,
+// 18.2 us with the 64 registers of 1024 threads, 16.9 with 80.
 template <typename T>
 struct ClusterLaunch {
     void (*kern)(const ClusterArgs<T>);
@@ -1418,7 +1421,7 @@ ClusterLaunch<T> cluster_launch(const lbm_batch *b, int cluster, int threads, si
                 need = std::max(need, sizeof(float) * sh.floats(ny, ny > 2 * FK));
             }
             const int t = (groups + 31) / 32 * 32;
-            return {t <= 512 ? cluster_vec_kernel<512> : cluster_vec_kernel<1024>, t, need};
+            return {t <= 512 ? cluster_vec_kernel<512, 2> : cluster_vec_kernel<768, 1>, t, need};
         }
     }
     return {cluster_batch_kernel<T>, threads, smem};

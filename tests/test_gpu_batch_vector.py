@@ -89,3 +89,19 @@ def test_every_grid_shape_is_taken_and_survives_other_batches():
             out.append(np.concatenate([f.ravel() for f in b.get_f()]))
     for o in out[1:]:
         assert np.array_equal(o, out[0])
+
+
+@pytest.mark.parametrize("nx,ny", [(512, 8), (520, 8), (756, 8), (58, 96)])
+def test_cluster_of_each_thread_count_is_the_grid_form(nx, ny):
+    # two CTAs of 512 | 520 threads, where the kernel changes, 760 and 768, the most that
+    # a slice can have
+    gp, _, f = make(nx, ny, "cs", "sc", 0.9)
+    out = []
+    for choose in (lambda b: b.set_launch(256, 1), lambda b: b.set_cluster(2, 512)):
+        with lbm.Batch([gp, gp]) as b:
+            choose(b)
+            b.set_f([f, f])
+            b.step(3)
+            b.sync()
+            out.append(np.stack(b.get_f()))
+    assert np.array_equal(out[0], out[1])
