@@ -19,10 +19,10 @@
 // most 8 rows) or 32 x 16.  The tile's populations are copied into shared memory
 // once per step (cp.async, at the step's start) and serve both phases when every
 // group has one tile; with several, phase B starts with the one that phase A ended
-// with.  Phase B stages the field with its halo, takes d/dx of the four cells from one 60-value window in recurrence form on packed pairs
-// (hdm_window4_paired, as the single-pass kernel does), d/dy likewise from windows
-// of the columns or, on short columns, from the folded weights, and collides the
-// four cells as two packed pairs.  Every other batch (FP64, or with a CDM lattice,
+// with.  Phase B stages the field with its halo, takes d/dx of the four cells from
+// one 60-value window in recurrence form on packed pairs (hdm_window4_paired, as the
+// single-pass kernel does), d/dy likewise from windows of the columns or, on short
+// columns, from the folded weights, and collides the four cells as two packed pairs.  Every other batch (FP64, or with a CDM lattice,
 // another radius or a narrower row in it) takes the form this replaced: one cell a
 // thread, 26 + 26 (40 + 40) taps loaded one by one.  us per step, per-cell form ->
 // vector path: twenty 200^2 lattices in the grid form 86.9 -> 28.4 (waiting per
