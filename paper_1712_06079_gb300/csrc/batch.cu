@@ -897,14 +897,19 @@ __device__ __forceinline__ void cluster_vec_steps(const ClusterArgs<float> &a, c
     const float *Re = gx == sl.ngw - 1 ? cluster.map_shared_rank(F, right) : F + xs + 4;
     const int up = (y + 1 >= ny ? 0 : y + 1) * sh.wf, here = y * sh.wf, down = (y == 0 ? ny - 1 : y - 1) * sh.wf;
     float *pr = ph + y * sh.wp + XH + xs;
-    // the field 28 columns to each side: element k of the halo, and where its rank holds it
-    const int nhalo = ny * 2 * XH;
-    auto halo = [&](int k, float *&dst, const float *&src) {
-        const int ry = k / (2 * XH), j = k - ry * (2 * XH);
-        const int xx = j < XH ? x0 - XH + j : x0 + w + j - XH;
+    // the field 28 columns to each side: element k of the halo, and where its rank holds
+    // it.  Where the row ends in part of a group, that group's window, laid out for four
+    // cells, reaches further: npad more columns, so that it reads what the grid form's
+    // ghost columns hold there
+    const int nhalo = ny * 2 * XH, npad = 4 * sl.ngw - w;
+    auto column = [&](int ry, int xx, float *&dst, const float *&src) {
         const int xg = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx), rk = sl.owner(xg);
         dst = ph + ry * sh.wp + XH + (xx - x0);
         src = cluster.map_shared_rank(ph + ry * sh.wp + XH + (xg - 4 * sl.group0(rk)), rk);
+    };
+    auto halo = [&](int k, float *&dst, const float *&src) {
+        const int ry = k / (2 * XH), j = k - ry * (2 * XH);
+        column(ry, j < XH ? x0 - XH + j : x0 + w + j - XH, dst, src);
     };
     float *hdst = ph;   // (the thread's first element, found once)
     const float *hsrc = ph;
@@ -948,6 +953,13 @@ __device__ __forceinline__ void cluster_vec_steps(const ClusterArgs<float> &a, c
             float *dst;
             const float *src;
             halo(k, dst, src);
+            *dst = *src;
+        }
+        for (int k = t; k < ny * npad; k += blockDim.x) {
+            const int ry = k / npad;
+            float *dst;
+            const float *src;
+            column(ry, x0 + w + XH + (k - ry * npad), dst, src);
             *dst = *src;
         }
         __syncthreads();
