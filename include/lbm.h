@@ -436,7 +436,9 @@ lbm_status lbm_step_noalloc(const lbm_params *p, const void *f_in, void *f_out);
  * allocation of the library fails as if the memory were exhausted (n = 0: all
  * of them); the failing call answers LBM_E_NOMEM and frees what it took, so a
  * test can walk every allocation of an entry point and check for leaks.  The
- * failure is made on the host; no GPU call fails. */
+ * failure is made on the host; no GPU call fails.  With LBM_DEBUG_FREE_BYTES=n
+ * set, lbm_adjoint_forward takes n bytes of device memory to be free when it
+ * decides how many further segments' records to keep. */
 lbm_status lbm_debug_alloc_stats(long long *live_device, long long *live_host);
 
 /* Test hook (not a passage of the paper) of the bounds-checked build, a

@@ -10,6 +10,10 @@
 // LBM_DEBUG_FAIL_ALLOC=n: once n allocations have succeeded since the
 // variable took its current value, every further allocation fails with
 // cudaErrorMemoryAllocation (n = 0: all of them).  Unset: no effect.
+//
+// LBM_DEBUG_FREE_BYTES=n: the device memory that the library takes to be free
+// where it bounds an allocation by that (the reverse mode's further records).
+// Unset: what the device reports.
 #include <cuda_runtime.h>
 
 #include <cstdlib>
@@ -90,6 +94,20 @@ cudaError_t host_alloc_raw(void **p, size_t bytes) {
         ++g_live_host;
     }
     return e;
+}
+
+size_t dev_free_bytes() {
+    if (const char *v = std::getenv("LBM_DEBUG_FREE_BYTES")) {
+        char *end = nullptr;
+        const long long n = std::strtoll(v, &end, 10);
+        if (end != v && n >= 0) return (size_t)n;
+    }
+    size_t free = 0, total = 0;
+    if (cudaMemGetInfo(&free, &total) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return free;
 }
 
 void dev_free(void *p) {

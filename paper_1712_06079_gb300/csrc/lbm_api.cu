@@ -98,7 +98,8 @@ lbm_status model_scalars(const lbm_params &p, ModelScalars *s) {
 constexpr int kTapeSlots = 2;
 static_assert(kTapeSlots >= 2, "the recompute runs at least one segment ahead");
 // Records of further segments that the forward keeps where memory allows, so that
-// the sweep need not recompute them: at most this many bytes per context.  144
+// the sweep need not recompute them: at most this many bytes per context, and half
+// of the device memory that is free once the rest of the tape is there.  144
 // steps at 512^2 (12 segments of 12) need 0.77 GB for all of them; a reverse step
 // costs 10.6 us with its record kept and 15.3 us beside a recompute.
 constexpr size_t kExtraTapeBytes = size_t(4) << 30;
@@ -634,18 +635,19 @@ lbm_status tape_forward(lbm_ctx *c, const T *rho0, int nsteps, int C, T *rhoT) {
                 free_tape(c);
                 return fail(c, LBM_E_NOMEM, "not enough device memory for the reverse sweep buffers");
             }
-            if (tape_rec(c)) {   // (done without if it cannot be had)
+            const int further = std::max(0, (nsteps - 1) / C - 1);   // segments before the last two
+            if (tape_rec(c) && further > 0) {
                 c->extra_rec = (sbytes + 255) / 256 * 256;
                 c->extra_q = (qbytes + 255) / 256 * 256;
                 const size_t per = (size_t)C * (c->extra_rec + c->extra_q);
-                const int want = (int)std::min<size_t>(std::max(0, (nsteps - 1) / C - 1), kExtraTapeBytes / per);
-                if (want > 0) {
+                size_t want = std::min<size_t>(further, std::min(kExtraTapeBytes, dev_free_bytes() / 2) / per);
+                for (; want > 0; want /= 2) {   // (fewer where that is refused, none at last)
                     if (dev_alloc(&c->extra, want * per) == cudaSuccess) {
-                        c->extra_segs = want;
-                    } else {
-                        cudaGetLastError();
-                        c->extra = nullptr;
+                        c->extra_segs = (int)want;
+                        break;
                     }
+                    cudaGetLastError();
+                    c->extra = nullptr;
                 }
             }
         }

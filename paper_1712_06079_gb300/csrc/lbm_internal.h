@@ -44,6 +44,8 @@ cudaError_t host_alloc(P **p, size_t bytes) {
     return host_alloc_raw((void **)p, bytes);
 }
 void dev_free(void *p);
+// Free device memory (0 if it cannot be asked for).
+size_t dev_free_bytes();
 void host_free(void *p);
 
 // f = f^eq(rho, u) (Eq. 2); ux/uy may be null (zero velocity).
