@@ -79,7 +79,11 @@
 // The MOM variant sweeps the state the same way but, instead of colliding,
 // writes rho (Eq. 3) and the half-step velocity of Eq. 11: 40 B in and 12 B out
 // per cell from the field the last step left, where the two-pass kernels'
-// moments read f twice and differentiate cell by cell.
+// moments read f twice and differentiate cell by cell.  What the step loses in the
+// rounding of its sums shows in these velocities, so the variant takes j from differences
+// of opposite populations (the 2048^2 CDM mixture: 7.8e-7 -> 5.0e-7 of the velocities'
+// rms against 64 bits, 5.4e-7 for the two-pass kernels), d/dy from sums of differences (see
+// column_phase) and correctly rounded quotients.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -364,6 +368,8 @@ __global__ void __launch_bounds__(NTHR, 2) fused_step_kernel(const __grid_consta
     // P's start P_(ys-2), over rows ys - 27 .. ys - 3 above the ring, and the
     // column's reference value q(ys - 1) come from the padded field, with all
     // loads in flight while the first copies land.
+    // MOM: the sums run over the differences of neighbouring rows instead (see there),
+    // and P starts one row further down.
     const bool fwdw = warp < SLAB / 2;
     const int cl = 32 * (warp & (SLAB / 2 - 1)) + lane;
     auto mag = [](float v) { return SC ? fabsf(v) : v; };   // the stencil's field value
@@ -371,16 +377,18 @@ __global__ void __launch_bounds__(NTHR, 2) fused_step_kernel(const __grid_consta
     if (!CDMG && cl < ncols) {
         const float *g = A.qin + x0 + QG - 4 + cl;
         const int yr = WALLS ? mirror_index(ys - 1, ny) : (ys - 1 < 0 ? ys - 1 + ny : ys - 1);
-        colref = mag(__ldg(g + (long long)yr * A.qpitch));
+        if (!MOM) colref = mag(__ldg(g + (long long)yr * A.qpitch));
         if (fwdw) {
-            float v[25];
+            constexpr int kRows = MOM ? 26 : 25;
+            float v[kRows];
 #pragma unroll
-            for (int k = 0; k < 25; ++k) {
+            for (int k = 0; k < kRows; ++k) {
                 const int y = ys - 27 + k;                  // ny >= 2 FK + 2 > 27: one wrap at most
                 v[k] = __ldg(g + (long long)(WALLS ? mirror_index(y, ny) : (y < 0 ? y + ny : y)) * A.qpitch);
             }
 #pragma unroll
-            for (int k = 0; k < 25; ++k) pcarry = fmaf(A.ry, pcarry, mag(v[k]) - colref);
+            for (int k = 0; k < 25; ++k)
+                pcarry = fmaf(A.ry, pcarry, MOM ? mag(v[MOM ? k + 1 : k]) - mag(v[k]) : mag(v[k]) - colref);
         }
     }
 
@@ -396,6 +404,13 @@ __global__ void __launch_bounds__(NTHR, 2) fused_step_kernel(const __grid_consta
     // chunks s .. s + 4 at a compile-time offset from that chunk's slot.  Slab
     // s + 1's recurrences run at the end of slab s, so one barrier per slab
     // serves them and the partial densities (and orders the far parts' reuse).
+    // MOM: a reference taken once per segment leaves each sum with the rounding of
+    // its largest deviation, which in a gas next to liquid is most of F / rho (the
+    // splash: 3.2e-6 of the rms of vy, 0.4e-6 from differences).  With
+    // d_i = q_(i+1) - q_i the same operator is
+    //   D_y = (w_1 + w_2 / (1 - r)) (q_(y+1) - q_(y-1)) + w_2 / (1 - r) (Q_(y+1) + P_(y-1)),
+    // P_y = d_(y-1) + r P_(y-1) and Q_y = d_y + r Q_(y+1): what is far off enters
+    // with its weight only, and P and Q add.
     auto column_phase = [&](int s) {
         // row Y0 + d of the slab (Y0 its first row, -1 <= d <= 33) is row e % 8 of ring
         // chunk s + e / 8, e = d + QBASE - 1
@@ -406,7 +421,9 @@ __global__ void __launch_bounds__(NTHR, 2) fused_step_kernel(const __grid_consta
             cb[j] = qn + slot * SLAB * NW + cl;
             slot = slot == QCH - 1 ? 0 : slot + 1;
         }
-        auto tq = [&](int d) { return mag(cb[(d + QBASE - 1) / SLAB][((d + QBASE - 1) % SLAB) * NW]) - colref; };
+        auto row = [&](int d) { return mag(cb[(d + QBASE - 1) / SLAB][((d + QBASE - 1) % SLAB) * NW]); };
+        auto tp = [&](int d) { return MOM ? row(d + 1) - row(d) : row(d) - colref; };   // row d's term of P
+        auto tq = [&](int d) { return MOM ? row(d) - row(d - 1) : row(d) - colref; };   // ... of Q
         float *buf = ab + (s & 1) * 2 * SLAB * NW + cl;
         const int bar_id = 1 + (warp & (SLAB / 2 - 1));
         if (fwdw) {
@@ -420,7 +437,7 @@ __global__ void __launch_bounds__(NTHR, 2) fused_step_kernel(const __grid_consta
 #pragma unroll
             for (int k = 0; k < SLAB; ++k) {
                 buf[k * NW] = v;                       // P_(Y0+k-1)
-                v = fmaf(A.ry, v, tq(k - 1));          // row Y0-1+k
+                v = fmaf(A.ry, v, tp(k - 1));          // row Y0-1+k
             }
             pcarry = v;   // P_(Y0+7) = P of the next slab's first row minus one
         } else {
@@ -482,6 +499,11 @@ __global__ void __launch_bounds__(NTHR, 2) fused_step_kernel(const __grid_consta
                 r2[h] = add2(add2(add2(v(0), v(2)), v(4)), add2(east, west));
                 jx2[h] = sub2(east, west);
                 jy2[h] = sub2(north, south);
+                if (MOM) {   // (opposite populations are close: their differences lose little)
+                    const float2 ne = sub2(v(5), v(7)), se = sub2(v(8), v(6));
+                    jx2[h] = add2(sub2(v(1), v(3)), add2(ne, se));
+                    jy2[h] = add2(sub2(v(2), v(4)), sub2(ne, se));
+                }
             }
             // for tau = 1 nothing after the moments reads f(t), so f(t) of the next
             // slab goes in flight here, across the derivatives and the collision
@@ -537,10 +559,11 @@ __global__ void __launch_bounds__(NTHR, 2) fused_step_kernel(const __grid_consta
                     const float *abs_ = ab + (s & 1) * 2 * SLAB * NW;
                     const float4 P = *reinterpret_cast<const float4 *>(abs_ + warp * NW + 4 * lane);
                     const float4 Q = *reinterpret_cast<const float4 *>(abs_ + (SLAB + warp) * NW + 4 * lane);
-                    dy[0] = fmaf(A.w1y, mag(qa.x) - mag(qb.x), A.w2y * (Q.x - P.x));
-                    dy[1] = fmaf(A.w1y, mag(qa.y) - mag(qb.y), A.w2y * (Q.y - P.y));
-                    dy[2] = fmaf(A.w1y, mag(qa.z) - mag(qb.z), A.w2y * (Q.z - P.z));
-                    dy[3] = fmaf(A.w1y, mag(qa.w) - mag(qb.w), A.w2y * (Q.w - P.w));
+                    auto both = [](float q, float p) { return MOM ? q + p : q - p; };
+                    dy[0] = fmaf(A.w1y, mag(qa.x) - mag(qb.x), A.w2y * both(Q.x, P.x));
+                    dy[1] = fmaf(A.w1y, mag(qa.y) - mag(qb.y), A.w2y * both(Q.y, P.y));
+                    dy[2] = fmaf(A.w1y, mag(qa.z) - mag(qb.z), A.w2y * both(Q.z, P.z));
+                    dy[3] = fmaf(A.w1y, mag(qa.w) - mag(qb.w), A.w2y * both(Q.w, P.w));
                 }
             }
             if constexpr (TAPE) {   // the record of f(t) at the lane's 4 cells of an own row
@@ -579,9 +602,9 @@ __global__ void __launch_bounds__(NTHR, 2) fused_step_kernel(const __grid_consta
                     for (int h = 0; h < 2; ++h) {
                         float2 Fx, Fy;
                         force2(h, Fx, Fy);
-                        const float2 inv = make_float2(__fdividef(1.0f, r2[h].x), __fdividef(1.0f, r2[h].y));
-                        v2[h] = mul2(fma2(splat2(0.5f), Fx, jx2[h]), inv);
-                        w2[h] = mul2(fma2(splat2(0.5f), Fy, jy2[h]), inv);
+                        const float2 nx2 = fma2(splat2(0.5f), Fx, jx2[h]), ny2 = fma2(splat2(0.5f), Fy, jy2[h]);
+                        v2[h] = make_float2(__fdiv_rn(nx2.x, r2[h].x), __fdiv_rn(nx2.y, r2[h].y));
+                        w2[h] = make_float2(__fdiv_rn(ny2.x, r2[h].x), __fdiv_rn(ny2.y, r2[h].y));
                     }
                     const long long o = (long long)yc * nx + xg;
                     auto put = [&](float *p, const float2 (&v)[2]) {
@@ -895,6 +918,9 @@ cudaError_t launch_sweep(void (*kern)(const FusedArgs), const FusedArgs &a, cuda
 cudaError_t launch_fused_moments(const Model<float> &m, bool sc, bool cdm, const float *f, const float *qin, float *rho,
                                  float *vx, float *vy, int *err, int seg_rows, cudaStream_t s, bool rev) {
     FusedArgs a = fused_args(m, f, qin, err, seg_rows, rev);
+    const double tail = m.wy[2] / (1.0 - 0.5 * (std::sqrt(5.0) - 3.0));   // w_2 / (1 - r)
+    a.w1y = (float)(m.wy[1] + tail);
+    a.w2y = (float)tail;
     a.mom[0] = rho;
     a.mom[1] = vx;
     a.mom[2] = vy;
