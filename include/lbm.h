@@ -416,7 +416,7 @@ void lbm_batch_destroy(lbm_batch *b);
  * The step is lbm_step's two-pass form (for LBM_F32: FP32 distributions,
  * FP64 arithmetic).  Its potential field (FP64 in both precisions) and the
  * error word live in a file-scope device array of LBM_STATIC_SCRATCH_BYTES
- * (4 MiB), the HDM's block sums in a second one (3 MiB); every GPU loading the
+ * (4 MiB), the HDM's block sums in a second one (4.5 MiB); every GPU loading the
  * library holds both until the process exits, so nx*ny may be at most (4 MiB - 256 B) / 8 = 524,256 cells; larger
  * lattices are rejected with LBM_E_INVALID before any device work.  The first call on a
  * device looks the arrays' device addresses up (with that device current), so

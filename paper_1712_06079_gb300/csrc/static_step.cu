@@ -23,7 +23,7 @@ static __device__ __align__(256) unsigned char g_static_scratch[LBM_STATIC_SCRAT
 // Block sums of the potential field (wide_step.cu); a lattice whose sums do not
 // fit (under 4 cells one way and close to the size limit) takes the direct
 // stencil instead.
-constexpr size_t kSumsBytes = 3u << 20;
+constexpr size_t kSumsBytes = 9u << 19;   // (4.5 MiB)
 static __device__ __align__(256) unsigned char g_static_sums[kSumsBytes];
 
 constexpr int kMaxDevices = 64;

@@ -18,6 +18,11 @@
 //   values that enter it (5 multiply-adds for the 40 cells past which r^j is
 //   below FP64 rounding, 1.9e-17) and steps S and T through the block, one
 //   multiply-add per cell each.
+// On a line of equal values T and S are equal up to rounding only, where the direct
+// form's differences vanish.  So that such a line has no derivative bit for bit (a
+// uniform lattice at rest stays at rest, a slab uniform along y stays so), pass 1 also
+// writes each block's value where its cells are equal, and pass 2 drops T - S where the
+// blocks around a cell all have that value: comparisons of bits, beside the FP64 work.
 // No halo of 40 cells is staged and no line is walked from its start.  Lines
 // whose length is no multiple of 8 end in a shorter block; with walls in y
 // (Sec. 5.5) the blocks continue in mirrored order, a mirrored block's BS being
@@ -38,7 +43,7 @@
 // beside each other), and 14.4 without programmatic launches.
 //
 // Measured, us per step (direct stencil before -> block sums): FP64 128^2 100 ->
-// 9.7, FP32 1024 x 8 35 -> 10.5; at 1024^2 pass 1 takes 92 and pass 2 159, i.e. 53
+// 9.1, FP32 1024 x 8 35 -> 9.4; at 1024^2 pass 1 takes 92 and pass 2 152, i.e. 53
 // and 92 FP64 instructions at one per 64 cycles and unit, which is the bound
 // there; small lattices are left with the latency of two dependent grids.
 #include <cuda_runtime.h>
@@ -67,66 +72,41 @@ struct WideArgs {
     int nbx, nby;            // blocks per row, per column
     int kbx, kby;            // blocks that cover kReach cells, wherever they start
     int ntx;                 // tiles per row of tiles
-    double *ys, *yt, *xs, *xt;   // block sums: ys, yt[by * nx + x]; xs, xt[y * nbx + bx]
+    // block sums BS, BT and the value of blocks of equal cells (else a NaN): y.[by * nx + x], x.[y * nbx + bx]
+    double *ys, *yt, *ye, *xs, *xt, *xe;
     int early;                   // the next grid is let in at the top (see spread)
-    long long nys, nxs;      // entries of each pair
+    long long nys, nxs;      // entries of each
 };
 
-// The block k of a line of nb blocks, k any integer: periodic, or (mirror) the
-// line continued by its mirror image, where a block's sums swap roles.
-template <bool MIRROR>
-__device__ __forceinline__ int block_of(int k, int nb, bool &swapped) {
-    if (MIRROR) {
-        const int p = 2 * nb;
-        int i = k % p;
-        if (i < 0) i += p;
-        swapped = i >= nb;
-        return swapped ? p - 1 - i : i;
+// Steps through the blocks of a line of nb, from block b on in direction dir: periodic,
+// or (mirror) the line continued by its mirror image, where a block's sums swap roles.
+struct BlockWalk {
+    int i, dir, nb;
+    bool mirror, swapped = false;
+    __device__ __forceinline__ void next() {
+        const int k = i + dir;
+        if (k >= 0 && k < nb) i = k;
+        else if (!mirror) i = k < 0 ? nb - 1 : 0;
+        else {
+            dir = -dir;
+            swapped = !swapped;
+        }
     }
-    swapped = false;
-    if (k >= 0 && k < nb) return k;
-    k %= nb;
-    return k < 0 ? k + nb : k;
-}
+};
 
-// The one-sided sum that enters block b of a line from below (dir = -1: S at
-// the cell before the block, from the blocks b - 1, b - 2, ...) or above (dir =
-// 1: T at the cell after it): kb blocks joined, the farthest first.  own / other:
-// the line's BS and BT for dir = -1, BT and BS for dir = 1 (stride between blocks).
-template <bool MIRROR>
-__device__ __forceinline__ double carry_into(const double *own, const double *other, long long stride, int b, int dir,
-                                             int nb, int kb, double r8, double rl, long long n, int *err) {
-    auto sum_of = [&](int k, bool &last) {
-        bool sw;
-        const int i = block_of<MIRROR>(b + dir * k, nb, sw);
-        last = i == nb - 1;
-        return in_bounds(i * stride, n, err) ? (MIRROR && sw ? other : own)[i * stride] : 0.0;
-    };
-    double acc = 0.0;
-    if (kb <= kJoin) {
-        double v[kJoin];
-        bool last[kJoin];
+// The value of the n cells at s if they are equal and finite, else a NaN (by the bits: a
+// comparison takes an FP64 slot).
+__device__ __forceinline__ double value_of_equal(const double *s, int step, int n) {
+    const long long v = __double_as_longlong(s[0]);
+    bool same = (v & 0x7ff0000000000000LL) != 0x7ff0000000000000LL;
 #pragma unroll
-        for (int k = 0; k < kJoin; ++k) {
-            v[k] = 0.0;
-            last[k] = false;
-            if (k < kb) v[k] = sum_of(k + 1, last[k]);
-        }
-#pragma unroll
-        for (int k = kJoin - 1; k >= 0; --k)
-            if (k < kb) acc = fma(last[k] ? rl : r8, acc, v[k]);
-    } else {
-        for (int k = kb; k >= 1; --k) {
-            bool last;
-            const double v = sum_of(k, last);
-            acc = fma(last ? rl : r8, acc, v);
-        }
-    }
-    return acc;
+    for (int k = 1; k < BK; ++k) same &= k >= n || __double_as_longlong(s[k * step]) == v;
+    return __longlong_as_double(same ? v : 0x7ff8000000000000LL);
 }
 
 // Block sums of a tile's fields: of `col` along its columns (warp 0), of `row`
-// along its rows (warp 1); lanes 0 .. 15 form BS, 16 .. 31 BT.
+// along its rows (warp 1), lanes 0 .. 15 BS, 16 .. 31 BT; the values of blocks of equal
+// cells by warp 2 (lanes 0 .. 15 columns, 16 .. 31 rows).
 __device__ __forceinline__ void write_block_sums(const WideArgs &A, const double (&col_f)[TY][TX + 1],
                                                  const double (&row_f)[TY][TX + 1], int tx, int ty) {
     const int nx = A.m.nx, ny = A.m.ny, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -160,29 +140,77 @@ __device__ __forceinline__ void write_block_sums(const WideArgs &A, const double
             const long long o = (long long)yc * A.nbx + bx;
             if (in_bounds(o, A.nxs, A.m.chk)) (fwd ? A.xs : A.xt)[o] = a;
         }
+    } else if (warp == 2) {
+        const int xc = tx * TX + (lane & 15), yc = ty * TY + (lane & 7), b = (lane >> 3) & 1, bx = 2 * tx + b;
+        const int len = fwd ? min(BK, ny - ty * TY) : min(BK, nx - bx * BK);
+        if (fwd ? xc < nx : yc < ny && len > 0) {
+            const double v = value_of_equal(fwd ? &col_f[0][lane & 15] : &row_f[lane & 7][b * BK], fwd ? TX + 1 : 1, len);
+            const long long o = fwd ? (long long)ty * nx + xc : (long long)yc * A.nbx + bx;
+            if (in_bounds(o, fwd ? A.nys : A.nxs, A.m.chk)) (fwd ? A.ye : A.xe)[o] = v;
+        }
     }
 }
 
-// The sum that enters this thread's block (warp 0: a column's, lanes 0 .. 15 S
-// from below, 16 .. 31 T from above; warp 1: a row's, 8 rows x 2 blocks); 0 elsewhere.
+// What enters the tile's blocks, warp 0 its columns (lanes 0 .. 15 from below, 16 .. 31
+// from above), warp 1 its rows (8 rows x 2 blocks): the one-sided sum of the kb blocks on
+// that side (S at the cell before the block, T at the cell after it), the farthest joined
+// first, returned.  Warps 2 and 3, lane by lane the same blocks: into E[0] (columns)
+// and E[1] whether those of both sides have the block's own value throughout.  One code
+// path for all four, without divisions: a grid this short runs most of its code once per
+// SM, and waits for its fetch (128^2, a path per warp 10.8 us per step, this 9.1).
 template <bool WALLS>
-__device__ __forceinline__ double tile_carry(const WideArgs &A, int tx, int ty) {
+__device__ __forceinline__ double tile_join(const WideArgs &A, int tx, int ty, int (&E)[2][16]) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool fwd = lane < 16;
-    if (warp == 0) {
-        const int xc = tx * TX + (lane & 15);
-        if (xc < A.m.nx)
-            return carry_into<WALLS>((fwd ? A.ys : A.yt) + xc, (fwd ? A.yt : A.ys) + xc, A.m.nx, ty, fwd ? -1 : 1, A.nby,
-                                     A.kby, A.r8, A.ryl, A.nys - xc, A.m.chk);
-    } else if (warp == 1) {
-        const int yc = ty * TY + (lane & 7), bx = 2 * tx + ((lane >> 3) & 1);
-        if (yc < A.m.ny && bx < A.nbx) {
-            const long long o = (long long)yc * A.nbx;
-            return carry_into<false>((fwd ? A.xs : A.xt) + o, (fwd ? A.xt : A.xs) + o, 1, bx, fwd ? -1 : 1, A.nbx,
-                                     A.kbx, A.r8, A.rxl, A.nxs - o, A.m.chk);
+    const bool fwd = lane < 16, cols = (warp & 1) == 0, sums = warp < 2;
+    const int xc = tx * TX + (lane & 15), yc = ty * TY + (lane & 7), bx = 2 * tx + ((lane >> 3) & 1);
+    const int nb = cols ? A.nby : A.nbx, kb = cols ? A.kby : A.kbx, b = cols ? ty : bx;
+    const long long n = cols ? A.nys : A.nxs, o0 = cols ? xc : (long long)yc * A.nbx, stride = cols ? A.m.nx : 1;
+    const double *own = cols ? (fwd ? A.ys : A.yt) : (fwd ? A.xs : A.xt);
+    const double *other = fwd ? A.yt : A.ys;   // (columns only: rows are never mirrored)
+    if (!sums) own = other = cols ? A.ye : A.xe;
+    const double rl = cols ? A.ryl : A.rxl;
+    const bool valid = cols ? xc < A.m.nx : yc < A.m.ny && bx < A.nbx;
+    double acc = 0.0;
+    bool same = false;
+    if (valid) {
+        auto at = [&](const BlockWalk &w) {
+            const long long o = o0 + w.i * stride;
+            return in_bounds(o, n, A.m.chk) ? (WALLS && w.swapped ? other : own)[o] : 0.0;
+        };
+        BlockWalk w{b, fwd ? -1 : 1, nb, WALLS && cols};
+        const long long mine = __double_as_longlong(at(w));   // (of warps 2 and 3)
+        same = (mine & 0x7ff0000000000000LL) != 0x7ff0000000000000LL;
+        if (kb <= kJoin) {
+            double v[kJoin];
+            unsigned last = 0;
+#pragma unroll
+            for (int k = 0; k < kJoin; ++k) {
+                w.next();
+                v[k] = k < kb ? at(w) : 0.0;
+                last |= (w.i == nb - 1 ? 1u : 0u) << k;
+            }
+#pragma unroll
+            for (int k = kJoin - 1; k >= 0; --k) {
+                if (k >= kb) continue;
+                if (sums) acc = fma(last >> k & 1 ? rl : A.r8, acc, v[k]);
+                else same &= __double_as_longlong(v[k]) == mine;
+            }
+        } else {
+            // (lines so short that the cover takes more blocks: the farthest first, each found from the block)
+            for (int k = kb; k >= 1; --k) {
+                w = BlockWalk{b, fwd ? -1 : 1, nb, WALLS && cols};
+                for (int j = 0; j < k; ++j) w.next();
+                const double v = at(w);
+                acc = fma(w.i == nb - 1 ? rl : A.r8, acc, v);
+                same &= __double_as_longlong(v) == mine;
+            }
         }
     }
-    return 0.0;
+    if (!sums) {
+        const int both = __shfl_xor_sync(0xffffffffu, same ? 1 : 0, 16) & (same ? 1 : 0);
+        if (fwd) E[warp & 1][lane] = both;
+    }
+    return acc;
 }
 
 // S_(i-1) and T_(i+1) of a tile's cells.
@@ -265,6 +293,7 @@ __global__ void __launch_bounds__(NT) wide_collide_kernel(const __grid_constant_
     constexpr int QW = TX + 2, QH = TY + 2;
     __shared__ double Q[QH][QW];                          // q over the tile and one cell around it
     __shared__ TileSums M;
+    __shared__ int E[2][16];
     const Model<double> &m = A.m;
     const int nx = m.nx, ny = m.ny;
     const long long n = (long long)nx * ny;
@@ -277,19 +306,31 @@ __global__ void __launch_bounds__(NT) wide_collide_kernel(const __grid_constant_
     if (A.early) ptx::griddep_launch_dependents();
     ptx::griddep_wait();   // pass 1 has written q and the block sums
 
-    // the rows and columns of the tile's halo: periodic, or mirrored across a wall
-    for (int k = threadIdx.x; k < QH * QW; k += NT) {
-        const int ry = k / QW, rx = k - ry * QW;
+    // every load is issued before the first value is waited for; the rows and columns
+    // of the tile's halo: periodic, or mirrored across a wall
+    constexpr int kStage = (QH * QW + NT - 1) / NT;
+    double qv[kStage];
+#pragma unroll
+    for (int j = 0; j < kStage; ++j) {
+        const int k = threadIdx.x + j * NT, ry = k / QW, rx = k - ry * QW;
         const int gx = min(x0 - 1 + rx, nx), gy = min(y0 - 1 + ry, ny);
         const int px = gx < 0 ? nx - 1 : (gx == nx ? 0 : gx);
         const int py = gy < 0 ? (WALLS ? 0 : ny - 1) : (gy == ny ? (WALLS ? ny - 1 : 0) : gy);
         const long long g = (long long)py * nx + px;
-        Q[ry][rx] = in_bounds(g, n, m.chk) ? q[g] : 0.0;
+        qv[j] = k < QH * QW && in_bounds(g, n, m.chk) ? q[g] : 0.0;
     }
-    const double carry = HDM ? tile_carry<WALLS>(A, tx, ty) : 0.0;
+    TS fv[kQ];
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) fv[i] = in_bounds(i * n + c, kQ * n, m.chk) ? f[i * n + c] : TS(0);
+    const double carry = HDM ? tile_join<WALLS>(A, tx, ty, E) : 0.0;
+#pragma unroll
+    for (int j = 0; j < kStage; ++j) {
+        const int k = threadIdx.x + j * NT, ry = k / QW, rx = k - ry * QW;
+        if (k < QH * QW) Q[ry][rx] = qv[j];
+    }
     double fi[kQ];
 #pragma unroll
-    for (int i = 0; i < kQ; ++i) fi[i] = in_bounds(i * n + c, kQ * n, m.chk) ? (double)f[i * n + c] : 0.0;
+    for (int i = 0; i < kQ; ++i) fi[i] = (double)fv[i];
     __syncthreads();
     auto mag = [](double v) { return SC ? fabs(v) : v; };
     if (HDM) tile_step<SC>(A, tx, ty, carry, Q, Q, M);
@@ -305,8 +346,10 @@ __global__ void __launch_bounds__(NT) wide_collide_kernel(const __grid_constant_
     const double *p = &Q[ly + 1][lx + 1];
     double dx, dy;
     if (HDM) {
-        dx = fma(A.c1, mag(p[1]) - mag(p[-1]), A.cs * (M.XT[ly][lx] - M.XS[ly][lx]));
-        dy = fma(A.c1, mag(p[QW]) - mag(p[-QW]), A.cs * (M.YT[ly][lx] - M.YS[ly][lx]));
+        const double tx_s = E[1][ly + (lx & 8)] ? 0.0 : M.XT[ly][lx] - M.XS[ly][lx];
+        const double ty_s = E[0][lx] ? 0.0 : M.YT[ly][lx] - M.YS[ly][lx];
+        dx = fma(A.c1, mag(p[1]) - mag(p[-1]), A.cs * tx_s);
+        dy = fma(A.c1, mag(p[QW]) - mag(p[-QW]), A.cs * ty_s);
     } else {   // Eq. 15 times 1/c_s^2
         const double ne = mag(p[QW + 1]), nw = mag(p[QW - 1]), se = mag(p[-QW + 1]), sw = mag(p[-QW - 1]);
         dx = (1.0 / 3.0) * (mag(p[1]) - mag(p[-1])) + (1.0 / 12.0) * ((ne + se) - (nw + sw));
@@ -580,6 +623,7 @@ template <bool HDM, bool TAU1>
 __global__ void __launch_bounds__(NT) wide_adj_b_kernel(const __grid_constant__ WideAdjArgs a) {
     __shared__ double QX[TY + 2][TX + 2], QY[TY + 2][TX + 2];   // D_bar with one cell around the tile
     __shared__ TileSums M;
+    __shared__ int E[2][16];
     const WideArgs &A = a.w;
     const Model<double> &m = A.m;
     const int nx = m.nx, ny = m.ny;
@@ -591,16 +635,27 @@ __global__ void __launch_bounds__(NT) wide_adj_b_kernel(const __grid_constant__ 
     const long long c = (long long)yc * nx + xc;
     if (A.early) ptx::griddep_launch_dependents();
     ptx::griddep_wait();   // A's output
-    for (int k = threadIdx.x; k < (TY + 2) * (TX + 2); k += NT) {
-        const int ry = k / (TX + 2), rx = k - ry * (TX + 2);
+    constexpr int kCells = (TY + 2) * (TX + 2), kStage = (kCells + NT - 1) / NT;
+    double sx[kStage], sy[kStage];   // (every load before the first wait, as in pass 2)
+#pragma unroll
+    for (int j = 0; j < kStage; ++j) {
+        const int k = threadIdx.x + j * NT, ry = k / (TX + 2), rx = k - ry * (TX + 2);
         const int gx = min(tx * TX - 1 + rx, nx), gy = min(ty * TY - 1 + ry, ny);
         const long long o = (long long)(gy < 0 ? ny - 1 : (gy == ny ? 0 : gy)) * nx + (gx < 0 ? nx - 1 : (gx == nx ? 0 : gx));
-        QX[ry][rx] = in_bounds(o, n, m.chk) ? a.aux[o] : 0.0;
-        QY[ry][rx] = in_bounds(o, n, m.chk) ? a.aux[n + o] : 0.0;
+        const bool ok = k < kCells && in_bounds(o, n, m.chk);
+        sx[j] = ok ? a.aux[o] : 0.0;
+        sy[j] = ok ? a.aux[n + o] : 0.0;
     }
-    const double carry = HDM ? tile_carry<false>(A, tx, ty) : 0.0;
     auto aux = [&](int k) { return in_bounds(k * n + c, 7 * n, m.chk) ? a.aux[k * n + c] : 0.0; };
     const double rb0 = aux(2), kappa = aux(3), theta = aux(4);
+    const double carry = HDM ? tile_join<false>(A, tx, ty, E) : 0.0;
+#pragma unroll
+    for (int j = 0; j < kStage; ++j) {
+        const int k = threadIdx.x + j * NT, ry = k / (TX + 2), rx = k - ry * (TX + 2);
+        if (k >= kCells) continue;
+        QX[ry][rx] = sx[j];
+        QY[ry][rx] = sy[j];
+    }
     __syncthreads();
     if (HDM) {
         tile_step<false>(A, tx, ty, carry, QY, QX, M);
@@ -611,8 +666,9 @@ __global__ void __launch_bounds__(NT) wide_adj_b_kernel(const __grid_constant__ 
     constexpr int QW = TX + 2;
     double dd;   // Dx[D_bar_x] + Dy[D_bar_y]
     if (HDM) {
-        dd = fma(A.c1, (px[1] - px[-1]) + (py[QW] - py[-QW]),
-                 A.cs * ((M.XT[ly][lx] - M.XS[ly][lx]) + (M.YT[ly][lx] - M.YS[ly][lx])));
+        const double tx_s = E[1][ly + (lx & 8)] ? 0.0 : M.XT[ly][lx] - M.XS[ly][lx];
+        const double ty_s = E[0][lx] ? 0.0 : M.YT[ly][lx] - M.YS[ly][lx];
+        dd = fma(A.c1, (px[1] - px[-1]) + (py[QW] - py[-QW]), A.cs * (tx_s + ty_s));
     } else {
         dd = (1.0 / 3.0) * ((px[1] - px[-1]) + (py[QW] - py[-QW])) +
              (1.0 / 12.0) * (((px[QW + 1] + px[-QW + 1]) - (px[QW - 1] + px[-QW - 1])) +
@@ -680,8 +736,10 @@ WideArgs args_of(const Model<double> &m, double *sums) {
     a.nxs = (long long)a.nbx * m.ny;
     a.ys = sums;
     a.yt = a.ys + a.nys;
-    a.xs = a.yt + a.nys;
+    a.ye = a.yt + a.nys;
+    a.xs = a.ye + a.nys;
     a.xt = a.xs + a.nxs;
+    a.xe = a.xt + a.nxs;
     a.early = spread_smem((long long)a.ntx * a.nby, kSpread) > 0;
     return a;
 }
@@ -738,7 +796,7 @@ bool wide_step_supported(const lbm_params &p) {
 
 size_t wide_sums_bytes(int nx, int ny) {
     const long long nbx = (nx + BK - 1) / BK, nby = (ny + BK - 1) / BK;
-    return sizeof(double) * 2 * (size_t)(nby * nx + nbx * ny);
+    return sizeof(double) * 3 * (size_t)(nby * nx + nbx * ny);
 }
 
 template <typename TS>
