@@ -374,8 +374,10 @@ cudaError_t moments_into(lbm_ctx *c, TS *r, TS *vx, TS *vy) {
                 if (e != cudaSuccess) return e;
                 q = (const float *)c->q;
             }
-            return launch_fused_moments(mf, is_sc(c), is_cdm(c), f, q, r, vx, vy, c->err, seg_rows_of(c), c->stream,
-                                        c->fused_rev);
+            int rows = seg_rows_of(c);
+            if ((c->p.ny + rows - 1) / rows > 65535)   // (more segments than a grid takes: the step is refused, this need not be)
+                rows = fused_auto_seg_rows(c->p.nx, c->p.ny, c->num_sms, is_cdm(c));
+            return launch_fused_moments(mf, is_sc(c), is_cdm(c), f, q, r, vx, vy, c->err, rows, c->stream, c->fused_rev);
         }
         if (c->p.flags & LBM_FLAG_F32_ARITH) {
             Model<float> mf = model_of<float>(c);
