@@ -1458,10 +1458,18 @@ cudaLaunchConfig_t cluster_config(const lbm_batch *b, int cluster, int threads, 
 }
 
 // Prepare a cluster launch and check that at least one cluster of it can be
-// resident.  Returns 0 or an error message.
+// resident.  Returns 0 or an error message.  The kernel's limit of shared memory belongs
+// to the function, not to the batch: every batch sets it to all that a block may take, so
+// that none, on whatever thread, lowers it before another's launch.
 template <typename T>
 const char *configure_cluster(const lbm_batch *b, const ClusterLaunch<T> &L, int cluster) {
-    if (cudaFuncSetAttribute(L.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem) != cudaSuccess)
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa{};
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaFuncGetAttributes(&fa, L.kern) != cudaSuccess || L.smem + fa.sharedSizeBytes > (size_t)optin ||
+        cudaFuncSetAttribute(L.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes) !=
+            cudaSuccess)
         return "shared memory of the cluster form not available";
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = cluster_config<T>(b, cluster, L.threads, L.smem, attr);
@@ -1501,8 +1509,6 @@ cudaError_t enqueue(lbm_batch *b, int nsteps) {
             cfg.gridDim = dim3((unsigned)(G.cluster * G.count));
             cfg.stream = b->gstream[g];
             e = cudaStreamWaitEvent(b->gstream[g], b->gfork, 0);
-            // (the limit belongs to the function: another batch may have set it lower since)
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(L.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
             if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, L.kern, ca);
             if (e == cudaSuccess) e = cudaEventRecord(b->gjoin[g], b->gstream[g]);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->gjoin[g], 0);
@@ -1522,8 +1528,7 @@ cudaError_t enqueue(lbm_batch *b, int nsteps) {
         const auto L = cluster_launch<T>(b, b->cluster, b->cluster_threads, b->cluster_smem, every);
         cudaLaunchAttribute attr[1];
         cudaLaunchConfig_t cfg = cluster_config<T>(b, b->cluster, L.threads, L.smem, attr);
-        const cudaError_t e = cudaFuncSetAttribute(L.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
-        return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, L.kern, ca);
+        return cudaLaunchKernelEx(&cfg, L.kern, ca);
     }
     cudaError_t e = cudaMemsetAsync(b->bar, 0, sizeof(BarrierState), b->stream);
     if (e != cudaSuccess) return e;
