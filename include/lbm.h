@@ -334,8 +334,8 @@ lbm_status lbm_batch_moments(lbm_batch *b, double *rho, double *vx, double *vy);
 /* Launch shape of the persistent kernel: threads per block (128, 256 or 512)
  * and co-resident blocks per SM (up to 1280 threads per SM in FP32, 1152 in
  * FP64; a batch whose kernel needs more shared memory runs with the blocks that
- * are resident at once).  Selects the grid form (a cluster form set earlier, by lbm_batch_set_cluster or the tuner, is
- * dropped). */
+ * are resident at once, which lbm_batch_get_launch then reports).  Selects the grid form
+ * (a cluster form set earlier, by lbm_batch_set_cluster or the tuner, is dropped). */
 lbm_status lbm_batch_set_launch(lbm_batch *b, int block_threads, int blocks_per_sm);
 lbm_status lbm_batch_get_launch(lbm_batch *b, int *block_threads, int *grid_blocks);
 

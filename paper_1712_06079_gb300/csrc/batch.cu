@@ -1534,10 +1534,7 @@ cudaError_t enqueue(lbm_batch *b, int nsteps) {
     if (e != cudaSuccess) return e;
     BatchArgs<T> a = make_args<T>(b, nsteps);
     cudaLaunchConfig_t cfg{};
-    // (a cooperative launch: at most what is resident at once)
-    const int resident = max_blocks_per_sm<T>(b, b->block_threads) * sm_count();
-    if (resident < 1) return cudaErrorInvalidConfiguration;
-    cfg.gridDim = dim3(std::min(b->grid_blocks, resident));
+    cfg.gridDim = dim3(b->grid_blocks);   // (a cooperative launch: never more than is resident at once)
     cfg.blockDim = dim3(b->block_threads);
     cfg.dynamicSmemBytes = grid_smem(b, b->block_threads);
     cfg.stream = b->stream;
@@ -1760,8 +1757,10 @@ lbm_status lbm_batch_set_launch(lbm_batch *b, int block_threads, int blocks_per_
     const int maxb = (b->prec == LBM_F64 ? 1152 : 1280) / block_threads;
     if (blocks_per_sm < 1 || blocks_per_sm > maxb)
         return bfail(b, LBM_E_INVALID, "blocks_per_sm must be in [1, " + std::to_string(maxb) + "]");
+    const int resident = max_blocks_per_sm(b, block_threads);
+    if (resident < 1) return bfail(b, LBM_E_CUDA, "no block of this shape is resident");
     b->block_threads = block_threads;
-    b->grid_blocks = blocks_per_sm * sm_count();
+    b->grid_blocks = std::min(blocks_per_sm, resident) * sm_count();
     b->cluster = 0;   // an explicit grid shape selects the grid form
     return LBM_OK;
 }
