@@ -1062,10 +1062,10 @@ __device__ __forceinline__ bool find_cell(const Inst<T> *inst, const int *table,
     const int ii = table[cell / kTableGrain];
     if (ii < 0) return false;
     const Inst<T> &I = inst[ii];
-    const long long local = cell - I.off;
-    if (local >= (long long)I.m.nx * I.m.ny) return false;
-    const int y = (int)(local / I.m.nx);
-    entry = I.fo + (long long)y * I.P + (local - (long long)y * I.m.nx);
+    const int local = (int)(cell - I.off);   // (an instance has at most 2^30 cells and its padding)
+    if (local >= I.m.nx * I.m.ny) return false;
+    entry = I.fo + local;
+    if (I.P != I.m.nx) entry += (long long)(local / I.m.nx) * (I.P - I.m.nx);   // padded rows
     return true;
 }
 
