@@ -622,7 +622,9 @@ __device__ __forceinline__ void cell_force(const BatchArgs<T> &a, const T *f, co
     const Model<T> &m = I.m;
     const bool sc = I.sc != 0;
     const T *q = a.q + I.qo + I.qx;
-    auto q_at = [&](int xx, int yy) { return __ldcg(q + (long long)yy * I.QP + xx); };   // (written by other SMs: past L1)
+    // (written by other SMs before the barrier, whose acquire orders plain loads too: the taps
+    // of neighbouring cells overlap, and L1 serves them)
+    auto q_at = [&](int xx, int yy) { return q[(long long)yy * I.QP + xx]; };
     auto phi = [&](int xx, int yy) { return qabs(q_at(xx, yy), sc); };
     auto wrap1 = [](int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); };
     T dx, dy;
