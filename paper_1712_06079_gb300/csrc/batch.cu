@@ -858,6 +858,7 @@ __global__ void __launch_bounds__(1024) cluster_batch_kernel(const ClusterArgs<T
 // on each side; d/dx from a window of the staged row, d/dy from the folded weights
 // or from windows of the columns; collision as two packed pairs into the own
 // entries; cluster barrier.
+constexpr int kPieces = 2 * XH / 4 + 1;   // pieces of the field's halo per row (cluster_vec_steps)
 struct SliceShape {   // shared memory of a CTA (floats), for the widest slice of ngm groups
     int ngm, wf, wp;  // groups; row pitch of a population, of the field
     __host__ __device__ SliceShape(int nx, int C) : ngm(((nx + 3) / 4 + C - 1) / C), wf(4 * ngm), wp(4 * ngm + 2 * XH) {}
@@ -878,8 +879,60 @@ struct Slice {
     __device__ int owner(int x) const { return ((x / 4 + 1) * C - 1) / ng; }   // rank of column x
 };
 
+// The field's halo, 28 columns to each side, in pieces of four columns: of each row 7 on
+// the left and 7 on the right, from the end of the last group, and the columns that a
+// shorter last group lacks (its window, laid out for four cells, reads what the grid
+// form's ghost columns hold there).  A piece lies in a run of some rank's columns, or ends
+// in the next rank's; in row 0 that of piece j:
+struct Piece {
+    const float *src, *src2;   // its first column, and column 0 of the next rank less `have`
+    int col, n, have;          // first column in this rank's rows, length, columns of the first run
+    int whole;                 // four columns on 16 bytes
+};
+__device__ __forceinline__ Piece piece_of(float *ph, const Slice &sl, int j) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int nx = sl.nx;
+    Piece p;
+    p.col = j < XH / 4 ? 4 * j - XH : (j < XH / 2 ? 4 * (sl.ngw + j) - XH : sl.w);
+    p.n = j < XH / 2 ? 4 : 4 * sl.ngw - sl.w;
+    const int xx = sl.x0 + p.col, xg = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx), rk = sl.owner(xg);
+    const int next = rk + 1 == sl.C ? 0 : rk + 1;
+    p.have = min(p.n, (next == 0 ? nx : 4 * sl.group0(next)) - xg);
+    p.whole = p.n == 4 && p.have == 4 && (xg & 3) == 0;
+    p.src = cluster.map_shared_rank(ph + XH + (xg - 4 * sl.group0(rk)), rk);
+    p.src2 = cluster.map_shared_rank(ph + XH, next) - p.have;
+    return p;
+}
+// The copies of a step, every row by the pieces of row 0.  Column by column, with the
+// place of all but a thread's first found again in every step, short slices took seven rounds;
+// and a call of its own, so that its few values do not spill those of the step (bytes of
+// spills in the four variants of 64 registers 1148 -> 520).  us per step: 16 x (128 x 8)
+// 5.0 -> 4.0, 64 x (250 x 8) 5.8 -> 5.1, the 64-lattice sweep (grouped) 18.7 -> 17.0.
+__device__ __noinline__ void copy_halo(float *ph, int wp, int ny, const Piece *pieces) {
+    for (int k = threadIdx.x; k < ny * kPieces; k += blockDim.x) {
+        const int ry = k / kPieces;
+        const Piece &p = pieces[k - ry * kPieces];
+        float *dst = ph + ry * wp + XH + p.col;
+        const float *src = p.src + ry * wp;
+        if (p.whole) {
+            *reinterpret_cast<float4 *>(dst) = *reinterpret_cast<const float4 *>(src);
+            continue;
+        }
+        const float *src2 = p.src2 + ry * wp;
+        const int n = p.n, have = p.have;
+        float v[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (c < n) v[c] = (c < have ? src : src2)[c];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (c < n) dst[c] = v[c];
+    }
+}
+
 template <bool SC, bool THIN>
-__device__ __forceinline__ void cluster_vec_steps(const ClusterArgs<float> &a, const Inst<float> &I, float *F) {
+__device__ __forceinline__ void cluster_vec_steps(const ClusterArgs<float> &a, const Inst<float> &I, float *F, Piece *pieces) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     const Model<float> &m = I.m;
@@ -899,23 +952,7 @@ __device__ __forceinline__ void cluster_vec_steps(const ClusterArgs<float> &a, c
     const float *Re = gx == sl.ngw - 1 ? cluster.map_shared_rank(F, right) : F + xs + 4;
     const int up = (y + 1 >= ny ? 0 : y + 1) * sh.wf, here = y * sh.wf, down = (y == 0 ? ny - 1 : y - 1) * sh.wf;
     float *pr = ph + y * sh.wp + XH + xs;
-    // the field 28 columns to each side: element k of the halo, and where its rank holds
-    // it.  Where the row ends in part of a group, that group's window, laid out for four
-    // cells, reaches further: npad more columns, so that it reads what the grid form's
-    // ghost columns hold there
-    const int nhalo = ny * 2 * XH, npad = 4 * sl.ngw - w;
-    auto column = [&](int ry, int xx, float *&dst, const float *&src) {
-        const int xg = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx), rk = sl.owner(xg);
-        dst = ph + ry * sh.wp + XH + (xx - x0);
-        src = cluster.map_shared_rank(ph + ry * sh.wp + XH + (xg - 4 * sl.group0(rk)), rk);
-    };
-    auto halo = [&](int k, float *&dst, const float *&src) {
-        const int ry = k / (2 * XH), j = k - ry * (2 * XH);
-        column(ry, j < XH ? x0 - XH + j : x0 + w + j - XH, dst, src);
-    };
-    float *hdst = ph;   // (the thread's first element, found once)
-    const float *hsrc = ph;
-    if (t < nhalo) halo(t, hdst, hsrc);
+    if (t < kPieces) pieces[t] = piece_of(ph, sl, t);   // (read after the first step's cluster barrier)
 
     for (int step = 0; step < a.nsteps; ++step) {
         float4 f4[kQ];
@@ -950,20 +987,7 @@ __device__ __forceinline__ void cluster_vec_steps(const ClusterArgs<float> &a, c
         if (valid)
 #pragma unroll
             for (int i = 0; i < kQ; ++i) *reinterpret_cast<float4 *>(F + i * plane + here + xs) = f4[i];
-        if (t < nhalo) *hdst = *hsrc;
-        for (int k = t + blockDim.x; k < nhalo; k += blockDim.x) {
-            float *dst;
-            const float *src;
-            halo(k, dst, src);
-            *dst = *src;
-        }
-        for (int k = t; k < ny * npad; k += blockDim.x) {
-            const int ry = k / npad;
-            float *dst;
-            const float *src;
-            column(ry, x0 + w + XH + (k - ry * npad), dst, src);
-            *dst = *src;
-        }
+        copy_halo(ph, sh.wp, ny, pieces);
         __syncthreads();
         float dx[4], dy[4], qc[4];
         if (THIN || m.ky != FK) {
@@ -1021,6 +1045,7 @@ __global__ void __launch_bounds__(MAXT, PER) cluster_vec_kernel(const ClusterArg
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ Piece pieces[kPieces];
     float *F = reinterpret_cast<float *>(smem_raw);
     const Inst<float> &I = a.inst[a.order[blockIdx.x / cluster.num_blocks()]];
     const int nx = I.m.nx, ny = I.m.ny;
@@ -1045,8 +1070,8 @@ __global__ void __launch_bounds__(MAXT, PER) cluster_vec_kernel(const ClusterArg
             if (in_bounds(i * a.nplane + g, kQ * a.nplane, I.m.chk)) *source(i, xl, y) = a.fin[i * a.nplane + g];
     }
     cluster.sync();
-    if (ny <= 8) I.sc ? cluster_vec_steps<true, true>(a, I, F) : cluster_vec_steps<false, true>(a, I, F);
-    else I.sc ? cluster_vec_steps<true, false>(a, I, F) : cluster_vec_steps<false, false>(a, I, F);
+    if (ny <= 8) I.sc ? cluster_vec_steps<true, true>(a, I, F, pieces) : cluster_vec_steps<false, true>(a, I, F, pieces);
+    else I.sc ? cluster_vec_steps<true, false>(a, I, F, pieces) : cluster_vec_steps<false, false>(a, I, F, pieces);
     for (int c = threadIdx.x; c < ny * sl.w; c += blockDim.x) {
         const int y = c / sl.w, xl = c - y * sl.w;
         const long long g = I.fo + (long long)y * I.P + sl.x0 + xl;
@@ -1408,7 +1433,8 @@ size_t cluster_smem_bytes(const lbm_batch *b, int cluster) {
 
 // Launch of the cluster form over the instances picked by `in`: kernel, threads
 // per CTA and shared memory.  The vector path's kernel takes a thread per group of
-// four cells of its widest slice whatever `threads` asks (a slice that
+// four cells of its widest slice whatever `threads` asks, and one per piece of the halo
+// up to 128 (each further round of copies from other ranks takes 0.35 us) (a slice that
 // cluster_smem_bytes admits has at most 768 of them, and never more shared memory than
 // that).  Up to 512 threads two CTAs share an SM, which with 64 registers and 650 bytes
 // of spills measured 18.8 us per step of the 64-lattice sweep (one cluster size) against
@@ -1425,16 +1451,17 @@ template <typename T, typename In>
 ClusterLaunch<T> cluster_launch(const lbm_batch *b, int cluster, int threads, size_t smem, In in) {
     if constexpr (sizeof(T) == 4) {
         if (b->vec) {
-            int groups = 0;
+            int groups = 0, pieces = 0;
             size_t need = 0;
             for (int i = 0; i < b->n; ++i) {
                 const int nx = b->params[i].nx, ny = b->params[i].ny;
                 if (!in(i)) continue;
                 const SliceShape sh(nx, cluster);
                 groups = std::max(groups, sh.ngm * ny);
+                pieces = std::max(pieces, kPieces * ny);
                 need = std::max(need, sizeof(float) * sh.floats(ny, ny > 2 * FK));
             }
-            const int t = (groups + 31) / 32 * 32;
+            const int t = (std::max(groups, std::min(pieces, 128)) + 31) / 32 * 32;
             return {t <= 512 ? cluster_vec_kernel<512, 2> : cluster_vec_kernel<768, 1>, t, need};
         }
     }
