@@ -331,6 +331,12 @@ __device__ __forceinline__ void group_sync(int g) {
 
 // ---- vector path ----
 
+// (LBM_CHECKED builds) the entries [o, o + n) lie in an array of `size` entries, shared
+// memory here: a rank's own or another's, which is laid out alike.
+__device__ __forceinline__ bool span_ok(long long o, int n, long long size, int *err) {
+    return in_bounds(o, size, err) && in_bounds(o + n - 1, size, err);
+}
+
 // A tile, four cells a thread: 64 x 8 on lattices of at most 8 rows (THIN), else
 // 32 x 16.
 template <bool THIN>
@@ -481,14 +487,25 @@ __device__ __forceinline__ void tile_gradient(const BatchArgs<float> &a, const I
     ptx::cp_async_wait_all();
     group_sync(g);
     const int row = t / GPR, gx = t % GPR;
+    const long long nY = (long long)yrows * TW;
+    // (the group's region holds the tile, and the window of d/dx lies in the staged row)
+    if (!in_bounds(kTileF + TH * XW + nY + (!THIN && ky == FK ? TH * TW : 0) - 1, tile_floats(ny), m.chk) ||
+        !span_ok(row * XW + 4 * gx, 60, TH * XW, m.chk)) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) dx[c] = dy[c] = qc[c] = 0.f;
+        return;
+    }
     bool folded = true;
     if constexpr (!THIN) {
         folded = ky != FK;
         if (!folded) {   // rows 4 rg .. 4 rg + 3 of a column each
-            const int col = t & 31, rg = t >> 5;
-            const float *w = Y + (4 * rg - 2) * TW + col;
+            const int col = t & 31, rg = t >> 5, w0 = (4 * rg - 2) * TW + col;
+            const float *w = Y + w0;
             float d[4];
-            window_derivative([&](int p) { return SC ? fabsf(w[p * TW]) : w[p * TW]; }, m.wy, a.r, a.r5, a.r25, d);
+            window_derivative([&](int p) {
+                const float u = in_bounds(w0 + p * TW, nY, m.chk) ? w[p * TW] : 0.f;
+                return SC ? fabsf(u) : u;
+            }, m.wy, a.r, a.r5, a.r25, d);
 #pragma unroll
             for (int c = 0; c < 4; ++c) D[(4 * rg + c) * TW + col] = d[c];
             group_sync(g);
@@ -496,7 +513,12 @@ __device__ __forceinline__ void tile_gradient(const BatchArgs<float> &a, const I
             dy[0] = v.x; dy[1] = v.y; dy[2] = v.z; dy[3] = v.w;
         }
     }
-    if (folded) folded_dy<SC, THIN>(Y + (row + ky) * TW + 4 * gx, TW, m, dy);
+    if (folded) {
+        if (span_ok(row * TW + 4 * gx, 2 * ky * TW + 4, nY, m.chk)) folded_dy<SC, THIN>(Y + (row + ky) * TW + 4 * gx, TW, m, dy);
+        else
+#pragma unroll
+            for (int c = 0; c < 4; ++c) dy[c] = 0.f;
+    }
     window_dx<SC>(X + row * XW + 4 * gx, m, a.r, a.r5, a.r25, dx, qc);
 }
 
@@ -889,7 +911,7 @@ struct Piece {
     int col, n, have;          // first column in this rank's rows, length, columns of the first run
     int whole;                 // four columns on 16 bytes
 };
-__device__ __forceinline__ Piece piece_of(float *ph, const Slice &sl, int j) {
+__device__ __forceinline__ Piece piece_of(float *ph, const Slice &sl, int j, int wp, int *err) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     const int nx = sl.nx;
@@ -902,6 +924,10 @@ __device__ __forceinline__ Piece piece_of(float *ph, const Slice &sl, int j) {
     p.whole = p.n == 4 && p.have == 4 && (xg & 3) == 0;
     p.src = cluster.map_shared_rank(ph + XH + (xg - 4 * sl.group0(rk)), rk);
     p.src2 = cluster.map_shared_rank(ph + XH, next) - p.have;
+    // (within the rows, here and there, whose pitch every rank shares; a row is one of ny)
+    if (p.n > 0 && !(span_ok(XH + p.col, p.n, wp, err) && span_ok(XH + xg - 4 * sl.group0(rk), p.have, wp, err) &&
+                     span_ok(XH, max(1, p.n - p.have), wp, err)))
+        p.n = p.whole = 0;
     return p;
 }
 // The copies of a step, every row by the pieces of row 0.  Column by column, with the
@@ -941,6 +967,7 @@ __device__ __forceinline__ void cluster_vec_steps(const ClusterArgs<float> &a, c
     const SliceShape sh(m.nx, sl.C);
     const int plane = ny * sh.wf, nx = sl.nx, x0 = sl.x0, w = sl.w;
     float *ph = F + kQ * plane, *D = ph + ny * sh.wp;
+    const int nF = kQ * plane, nP = ny * sh.wp, nD = ny * sh.wf;   // entries of each (checked build)
     const int left = sl.rank == 0 ? sl.C - 1 : sl.rank - 1, right = sl.rank == sl.C - 1 ? 0 : sl.rank + 1;
     const int t = threadIdx.x, row = t / sl.ngw, gx = t - row * sl.ngw, lane = t & 31;
     const bool valid = row < ny;
@@ -952,21 +979,22 @@ __device__ __forceinline__ void cluster_vec_steps(const ClusterArgs<float> &a, c
     const float *Re = gx == sl.ngw - 1 ? cluster.map_shared_rank(F, right) : F + xs + 4;
     const int up = (y + 1 >= ny ? 0 : y + 1) * sh.wf, here = y * sh.wf, down = (y == 0 ? ny - 1 : y - 1) * sh.wf;
     float *pr = ph + y * sh.wp + XH + xs;
-    if (t < kPieces) pieces[t] = piece_of(ph, sl, t);   // (read after the first step's cluster barrier)
+    if (t < kPieces) pieces[t] = piece_of(ph, sl, t, sh.wp, m.chk);   // (read after the first step's cluster barrier)
 
     for (int step = 0; step < a.nsteps; ++step) {
         float4 f4[kQ];
 #pragma unroll
         for (int i = 0; i < kQ; ++i) {   // f_i(x) = post_i(x - e_i)
             const int o = i * plane + (ey(i) == 1 ? down : (ey(i) == -1 ? up : here));
-            float4 v = *reinterpret_cast<const float4 *>(F + o + xs);
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (span_ok(o + xs, 4, nF, m.chk)) v = *reinterpret_cast<const float4 *>(F + o + xs);
             if (ex(i) == 1) {
                 float l = __shfl_up_sync(0xffffffffu, v.w, 1);
-                if (first) l = Le[o];
+                if (first && in_bounds(o + (gx == 0 ? wl : xs) - 1, nF, m.chk)) l = Le[o];
                 v = make_float4(l, v.x, v.y, v.z);
             } else if (ex(i) == -1) {
                 float r = __shfl_down_sync(0xffffffffu, v.x, 1);
-                if (last) r = Re[o];
+                if (last && in_bounds(o + (gx == sl.ngw - 1 ? 0 : xs + 4), nF, m.chk)) r = Re[o];
                 v = make_float4(v.y, v.z, v.w, r);
                 if (nc == 1) v.x = r;   // (a row's shorter last group)
                 if (nc == 2) v.y = r;
@@ -976,7 +1004,7 @@ __device__ __forceinline__ void cluster_vec_steps(const ClusterArgs<float> &a, c
         }
         float q[4];
         four_potentials(m, SC, f4, valid ? nc : 0, q, a.err);
-        if (valid) {
+        if (valid && span_ok(pr - ph, nc, nP, m.chk)) {
             if (nc == 4) *reinterpret_cast<float4 *>(pr) = make_float4(q[0], q[1], q[2], q[3]);
             else
 #pragma unroll
@@ -986,7 +1014,8 @@ __device__ __forceinline__ void cluster_vec_steps(const ClusterArgs<float> &a, c
         cluster.sync();   // every rank has pulled, and formed its field
         if (valid)
 #pragma unroll
-            for (int i = 0; i < kQ; ++i) *reinterpret_cast<float4 *>(F + i * plane + here + xs) = f4[i];
+            for (int i = 0; i < kQ; ++i)
+                if (span_ok(i * plane + here + xs, 4, nF, m.chk)) *reinterpret_cast<float4 *>(F + i * plane + here + xs) = f4[i];
         copy_halo(ph, sh.wp, ny, pieces);
         __syncthreads();
         float dx[4], dy[4], qc[4];
@@ -997,7 +1026,8 @@ __device__ __forceinline__ void cluster_vec_steps(const ClusterArgs<float> &a, c
             auto tap = [&](float wj) {   // (folded_dy on the wrapped rows)
                 yp = yp + 1 == ny ? 0 : yp + 1;
                 ym = ym == 0 ? ny - 1 : ym - 1;
-                folded_tap<SC>(wj, ph + yp * sh.wp + XH + xs, ph + ym * sh.wp + XH + xs, dy);
+                if (span_ok(yp * sh.wp + XH + xs, 4, nP, m.chk) && span_ok(ym * sh.wp + XH + xs, 4, nP, m.chk))
+                    folded_tap<SC>(wj, ph + yp * sh.wp + XH + xs, ph + ym * sh.wp + XH + xs, dy);
             };
             if constexpr (THIN) {
 #pragma unroll
@@ -1011,22 +1041,28 @@ __device__ __forceinline__ void cluster_vec_steps(const ClusterArgs<float> &a, c
                 const int rg = k / w, xl = k - rg * w;
                 float d[4];
                 window_derivative([&](int p) {
-                    const float u = ph[wrap_index(4 * rg - 28 + p, ny) * sh.wp + XH + xl];
+                    const int o = wrap_index(4 * rg - 28 + p, ny) * sh.wp + XH + xl;
+                    const float u = in_bounds(o, nP, m.chk) ? ph[o] : 0.f;
                     return SC ? fabsf(u) : u;
                 }, m.wy, a.r, a.r5, a.r25, d);
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
-                    if (4 * rg + c < ny) D[(4 * rg + c) * sh.wf + xl] = d[c];
+                    if (4 * rg + c < ny && in_bounds((4 * rg + c) * sh.wf + xl, nD, m.chk)) D[(4 * rg + c) * sh.wf + xl] = d[c];
             }
             __syncthreads();
-            const float4 d4 = *reinterpret_cast<const float4 *>(D + here + xs);
+            float4 d4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (span_ok(here + xs, 4, nD, m.chk)) d4 = *reinterpret_cast<const float4 *>(D + here + xs);
             dy[0] = d4.x; dy[1] = d4.y; dy[2] = d4.z; dy[3] = d4.w;
         }
-        window_dx<SC>(pr - XH, m, a.r, a.r5, a.r25, dx, qc);
+        if (span_ok(pr - XH - ph, 60, nP, m.chk)) window_dx<SC>(pr - XH, m, a.r, a.r5, a.r25, dx, qc);
+        else
+#pragma unroll
+            for (int c = 0; c < 4; ++c) dx[c] = qc[c] = 0.f;
         F2 post[2][kQ];
 #pragma unroll
         for (int i = 0; i < kQ; ++i) {
-            const float4 v4 = *reinterpret_cast<const float4 *>(F + i * plane + here + xs);
+            float4 v4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (span_ok(i * plane + here + xs, 4, nF, m.chk)) v4 = *reinterpret_cast<const float4 *>(F + i * plane + here + xs);
             post[0][i] = pair_of(v4, 0);
             post[1][i] = pair_of(v4, 1);
         }
@@ -1034,8 +1070,9 @@ __device__ __forceinline__ void cluster_vec_steps(const ClusterArgs<float> &a, c
         if (valid)
 #pragma unroll
             for (int i = 0; i < kQ; ++i)
-                *reinterpret_cast<float4 *>(F + i * plane + here + xs) =
-                    make_float4(post[0][i].v.x, post[0][i].v.y, post[1][i].v.x, post[1][i].v.y);
+                if (span_ok(i * plane + here + xs, 4, nF, m.chk))
+                    *reinterpret_cast<float4 *>(F + i * plane + here + xs) =
+                        make_float4(post[0][i].v.x, post[0][i].v.y, post[1][i].v.x, post[1][i].v.y);
         cluster.sync();
     }
 }
@@ -1057,7 +1094,8 @@ __global__ void __launch_bounds__(MAXT, PER) cluster_vec_kernel(const ClusterArg
     auto source = [&](int i, int xl, int y) {
         const int yy = y - ey(i) < 0 ? ny - 1 : (y - ey(i) >= ny ? 0 : y - ey(i)), xx = sl.x0 + xl - ex(i);
         const int xg = xx < 0 ? nx - 1 : (xx >= nx ? 0 : xx), rk = sl.owner(xg);
-        float *o = F + i * plane + yy * sh.wf + (xg - 4 * sl.group0(rk));
+        const int e = i * plane + yy * sh.wf + (xg - 4 * sl.group0(rk));
+        float *o = F + (in_bounds(e, (long long)kQ * plane, I.m.chk) ? e : 0);
         return rk == sl.rank ? o : cluster.map_shared_rank(o, rk);
     };
     for (int c = threadIdx.x; c < kQ * plane; c += blockDim.x) F[c] = 1.f;   // (columns past a shorter slice: computed on, dropped)
