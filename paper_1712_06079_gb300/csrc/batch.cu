@@ -27,9 +27,9 @@
 // thread, 26 + 26 (40 + 40) taps loaded one by one.  us per step, per-cell form ->
 // vector path: twenty 200^2 lattices in the grid form 86.9 -> 28.4 (waiting per
 // lattice and per group instead of for the whole grid was no faster, and neither was
-// starting the next tile's copy as soon as this one's populations are in registers; about
-// 1900 instructions per thread and step); the 64-lattice sweep (590,000 cells) 41.5 -> 23 in the
-// grid form, 31.8 -> 20.8 with one cluster size, 27.6 -> 16.9 as tuned (grouped).
+// starting the next tile's copy as soon as this one's populations are in registers; 1850
+// instructions per thread and step); the 64-lattice sweep (616,000 cells) 41.5 -> 23 in the
+// grid form, 31.8 -> 20.3 with one cluster size, 27.6 -> 17.0 as tuned (grouped).
 //
 // A cell's operations depend on its absolute position only (the groups of four
 // start at multiples of four), packed pairs round as single operations do, and
@@ -1475,7 +1475,7 @@ size_t cluster_smem_bytes(const lbm_batch *b, int cluster) {
 // up to 128 (each further round of copies from other ranks takes 0.35 us) (a slice that
 // cluster_smem_bytes admits has at most 768 of them, and never more shared memory than
 // that).  Up to 512 threads two CTAs share an SM, which with 64 registers and 650 bytes
-// of spills measured 18.8 us per step of the 64-lattice sweep (one cluster size) against
+// of spills (520 since the halo's copies are a call) measured 18.8 us per step of the 64-lattice sweep (one cluster size) against
 // 21.1 with one CTA of 118 registers.  Above that there is one CTA per SM in any case and
 // it may take 80 registers: as tuned, 34 + 12 of the 64 lattices in CTAs of 744 threads,
 // 18.2 us with the 64 registers of 1024 threads, 16.9 with 80.

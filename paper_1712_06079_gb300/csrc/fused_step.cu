@@ -827,7 +827,8 @@ int fused_q_pitch(int nx) { return nx + 2 * QG; }
 // most 9 slabs does (1024^2 19.1 -> 13.5 us), else the one before (2048^2 57.6 us at 126
 // rows against 58.5 at one wave of 17 slabs), with 62 rows for 126 where that makes
 // fewer wave-slabs (2048^2, 306 CTAs of 126 rows for 304 slots: 57.6 -> 54.1 us, tau 0.9
-// 59.8 -> 57.0; 4096^2 keeps 126: 220, at 62 rows 214, tau 0.9 225 and 226).
+// 59.8 -> 57.0).  That is not the best height everywhere: 4096^2 keeps 126 rows by it, 220
+// us, where 62 take 214 (tau 0.9: 225 and 226); the tuner finds it.
 int fused_auto_seg_rows(int nx, int ny, int num_sms, bool cdm) {
     const long long strips = (nx + TXI - 1) / TXI, slots = 2LL * num_sms;
     // slabs of the shortest segments that make at most `waves` full waves (0: none do)

@@ -43,9 +43,9 @@
 // beside each other), and 14.4 without programmatic launches.
 //
 // Measured, us per step (direct stencil before -> block sums): FP64 128^2 100 ->
-// 9.1, FP32 1024 x 8 35 -> 9.4; at 1024^2 pass 1 takes 92 and pass 2 152, i.e. 53
-// and 92 FP64 instructions at one per 64 cycles and unit, which is the bound
-// there; small lattices are left with the latency of two dependent grids.
+// 9.1, FP32 1024 x 8 35 -> 9.4, FP64 1024^2 -> 244, where one at a time pass 1 takes 91
+// and pass 2 159 with the FP64 units 80 and 83 % busy, which is the bound there;
+// small lattices are left with the latency of two dependent grids.
 #include <cuda_runtime.h>
 
 #include <algorithm>
